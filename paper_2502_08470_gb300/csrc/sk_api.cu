@@ -515,12 +515,13 @@ int plan_tape(const sk_paths* X, const sk_paths* Y, const sk_options* o, int T, 
     const int64_t pts = (o->flags & SK_FLAG_INCREMENTS) ? 0 : 1;
     const int64_t lx = std::max<int64_t>(X->max_len - pts, 1), ly = std::max<int64_t>(Y->max_len - pts, 1);
     int64_t rows = lx << lam;
-    const int64_t cols = ly << lam;
+    int64_t cols = ly << lam;
     int row;
     if (is_fd(o)) {
-        // FD: each lane sweeps 2^lambda node rows (one coarse row) over the refined columns
+        // FD: each lane sweeps 2^lambda node rows (one coarse row), fd_cols refined columns a step
         if (lam > 4) return fail(SK_ERR_UNSUPPORTED, "the FD adjoint supports dyadic orders 0..4");
         rows = lx;
+        cols /= fd_tape_cols(lam);
         row = fd_tape_row_elems(T, lam);
     } else {
         const bool interp = o->scheme == SK_POLY_INTERP;

@@ -25,6 +25,8 @@ const void* bwd_fd_tape_ptr(int T, int order, int lam) {
 
 int fd_tape_row_elems(int T, int lam) { return T ? fd_tape_row<float>(1 << lam) : fd_tape_row<double>(1 << lam); }
 
+int fd_tape_cols(int lam) { return fd_cols(1 << lam); }
+
 int bwd_fd_ring_bytes(int T, int lam) {
     switch (lam) {
         case 0: return T ? fd_ring_warp_bytes<float, 1>() : fd_ring_warp_bytes<double, 1>();

@@ -25,10 +25,11 @@ const void* fwd_approx_tape_ptr_f32_mt(int N);
 const void* fwd_approx_tape_ptr_f64(int N);
 const void* fwd_fd_kernel_ptr(int T, int order, int lam, bool coop, bool tape = false);
 // The FD forward that records the adjoint's tape, the FD adjoint from it (dyadic orders 0..4; NULL
-// otherwise), and the elements of one lane's tape row.
+// otherwise), the elements of one lane's tape row and the refined columns it covers.
 const void* fwd_fd_tape_ptr(int T, int order, int lam);
 const void* bwd_fd_tape_ptr(int T, int order, int lam);
 int fd_tape_row_elems(int T, int lam);
+int fd_tape_cols(int lam);  // refined columns per warp step
 // Shared memory of one warp of bwd_fd_tape_kernel (its ring of tape rows).
 int bwd_fd_ring_bytes(int T, int lam);
 const void* fwd_fd_coop_ptr(int T, int order, int lam);

@@ -20,10 +20,19 @@
 //
 // Parallel layout.  One warp owns one pair (or, for long pairs, a block of warps shares it with
 // one strip per warp in a pipeline, as in the polynomial wavefront).  Lane r owns R = min(2^lambda, 16) consecutive node
-// rows (a "row group"; all in one coarse row) and sweeps the refined columns; the top node of
-// its group moves one lane up per step by __shfl_up_sync, and lane 31's top nodes are handed to
-// lane 0 of the next strip through a per-warp buffer, as in the polynomial wavefront.  FP32 keeps
-// a power-of-two exponent per lane (rescale by 2^-64 / 2^64 outside [2^-64, 2^64]).
+// rows (a "row group"; all in one coarse row) and sweeps the refined columns, C = fd_cols(R) of them
+// (all in one coarse column) per warp step; the C top nodes of its group move one lane up per step
+// by __shfl_up_sync, and lane 31's top nodes are handed to lane 0 of the next strip through a
+// per-warp buffer, as in the polynomial wavefront.  FP32 keeps a power-of-two exponent per lane
+// (rescale by 2^-64 / 2^64 outside [2^-64, 2^64]).
+//
+// A sub-cell is six or seven instructions, so with one column per step the sweep is bound by
+// everything else a step does: exponents, shuffles, the inner product, index arithmetic and the
+// hand-off (209 issue slots per warp step of 4 sub-cells a lane at lambda = 2).  A step of R x C
+// sub-cells pays for these once and forms the one m they share once.  Measured: FD2, lambda = 2,
+// 128 x 128 Gram of 129-point paths, d = 8, FP32, 6.24 -> 2.87 ms with 4 columns a step, 170 warp
+// instructions a step at 0.76 issued a cycle: bound by issue.  FD2, lambda = 1, 48 x 48 pairs, forward
+// with tape and adjoint: 1.63 -> 1.02 ms with 2 columns a step, whose tape is half as long.
 #pragma once
 
 #include <type_traits>
@@ -33,13 +42,23 @@
 
 namespace sk {
 
-// One lane's row of the FD forward tape: its R node differences v (before the column's update),
-// k0 = k(gR, J), k1 = k(gR, J+1), the sub-cell m and the exponent, padded to 16 bytes.  From it the
-// adjoint rebuilds the lane's R sub-cells of column J (fd_tape_row elements per lane and step,
-// laid out [vector][lane] like the polynomial tapes).
+// Refined columns a lane takes per warp step: the coarse cell's own for 2 or 4 of them, else as many
+// as keep the tile's 16 to 32 sub-cells in registers.  A divisor of 2^lambda for R = min(2^lambda, 16),
+// so that the tile lies in one coarse cell.
+__host__ __device__ constexpr int fd_cols(int R) { return R <= 4 ? R : (R == 8 ? 4 : 2); }
+
+// |m| up to which a tile is swept without looking at the magnitudes between its columns: the update
+// then multiplies a node by less than 4, the longest chain of updates in a tile has R + C - 1 <= 17
+// of them, and values start within [2^-64, 2^64].  Above it the tile is rescaled after every column.
+constexpr float kFdTileM = 1.0f;
+
+// One lane's row of the FD forward tape: its R node differences v (before the tile's update), the
+// C + 1 bottom nodes k(gR, J .. J + C), the sub-cells' m and the exponent, padded to 16 bytes.  From
+// it the adjoint rebuilds the lane's R x C sub-cells (fd_tape_row elements per lane and step, laid
+// out [vector][lane] like the polynomial tapes).
 template <typename T>
 __host__ __device__ constexpr int fd_tape_row(int R) {
-    return ((R + 4) * static_cast<int>(sizeof(T)) + 15) / 16 * 16 / static_cast<int>(sizeof(T));
+    return ((R + fd_cols(R) + 3) * static_cast<int>(sizeof(T)) + 15) / 16 * 16 / static_cast<int>(sizeof(T));
 }
 
 template <typename T>
@@ -63,15 +82,16 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
     const T* __restrict__ incX = static_cast<const T*>(L.X.inc);
     const T* __restrict__ incY = static_cast<const T*>(L.Y.inc);
 
+    constexpr int C = fd_cols(R);
     const int lam = L.lam;
-    const int nI = static_cast<int>(P.lx << lam);   // refined node rows 0..nI
-    const int nJ = static_cast<int>(P.ly << lam);   // refined node columns 0..nJ
+    const int nI = static_cast<int>(P.lx << lam);       // refined node rows 0..nI
+    const int nJ = static_cast<int>(P.ly << lam) / C;   // tiles of C refined columns per row group
     const int groups = nI / R;
     // Period of a warp's strips.  Alone, a warp starts its next strip as soon as lane 0 is free
-    // (P = max(cols, 32)).  In a cooperative block that overlap can deadlock: a warp whose lane 0
+    // (P = max(tiles, 32)).  In a cooperative block that overlap can deadlock: a warp whose lane 0
     // waits on the ring of other warps also holds back its lanes still publishing the previous
     // strip, which those warps need.  A warp therefore starts strip k + 1 only after finishing
-    // strip k (P = cols + 31), unless the rows are longer than the ring's lag (cols > 31 CW),
+    // strip k (P = tiles + 31), unless the rows are longer than the ring's lag (tiles > 31 CW),
     // where the overlapped schedule keeps every wait pointed at finished work.  A model of this
     // schedule (tests/test_pipeline_schedule.py) checks the rule and the deadlock it avoids.
     const int period = CW == 1 ? (nJ > 32 ? nJ : 32) : (nJ > 31 * CW ? nJ : nJ + 31);
@@ -85,30 +105,36 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
     const T* xbase = incX + P.xs * dpad;
     const T* ybase = incY + P.ys * dpad;
 
-    T v[R];     // k(gR + 1 + r, jj) - k(gR + r, jj) for the lane's group g at its column jj
-    T kb_prev = T(1), top = T(0);
+    T v[R];     // k(gR + 1 + r, J) - k(gR + r, J) for the lane's group g at its tile's first column
+    T kb_prev = T(1), top[C];
     int ea = 0, eo = 0;
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = T(0);
-    int jj = -lane, sl = 0, gs = w;     // column, local strip, global strip
+#pragma unroll
+    for (int c = 0; c < C; ++c) top[c] = T(0);
+    int jj = -lane, sl = 0, gs = w;     // tile, local strip, global strip
     bool stuck = false;
 
     for (int step = 0; step < nsteps; ++step) {
-        T kb = __shfl_up_sync(kFull, top, 1);            // k(gR, jj + 1) from the lane below
+        T kb[C];                                             // k(gR, J + 1 .. J + C) from the lane below
+#pragma unroll
+        for (int c = 0; c < C; ++c) kb[c] = __shfl_up_sync(kFull, top[c], 1);
         int eb = kRescale ? __shfl_up_sync(kFull, eo, 1) : 0;
         const int g = (gs << 5) + lane;
         const bool active = jj >= 0 && jj < nJ && g < groups && sl < nloc;
         if (active) {
             if (lane == 0) {
-                if (gs == 0) {
-                    kb = T(1);                               // row 0: k(s_0, .) = 1
+                if (gs == 0) {                               // row 0: k(s_0, .) = 1
+#pragma unroll
+                    for (int c = 0; c < C; ++c) kb[c] = T(1);
                     eb = 0;
                 } else {
                     if constexpr (CW > 1) {
                         if (!stuck && !wait_progress(prog + (w + CW - 1) % CW, (gs - 1) * nJ + jj + 1, wait_polls(L)))
                             stuck = true;
                     }
-                    kb = hprev[jj];
+#pragma unroll
+                    for (int c = 0; c < C; ++c) kb[c] = hprev[jj * C + c];
                     if (kRescale) eb = eprev[jj];
                 }
             }
@@ -120,7 +146,9 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
             }
             if (kRescale && ea != eb) {
                 if (ea > eb) {
-                    kb *= (eb - ea < -126) ? T(0) : fd_pow2<T>(eb - ea);
+                    const T f = (eb - ea < -126) ? T(0) : fd_pow2<T>(eb - ea);
+#pragma unroll
+                    for (int c = 0; c < C; ++c) kb[c] *= f;
                 } else {
                     const T f = (ea - eb < -126) ? T(0) : fd_pow2<T>(ea - eb);
 #pragma unroll
@@ -130,8 +158,8 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
                 }
             }
             const T m = row_dot<T>(xbase + static_cast<int64_t>((g * R) >> lam) * dpad,
-                                   ybase + static_cast<int64_t>(jj >> lam) * dpad, L.nvec) * sub;
-            if constexpr (TAPE) {  // the column's inputs for the adjoint (fd_tape_row)
+                                   ybase + static_cast<int64_t>((jj * C) >> lam) * dpad, L.nvec) * sub;
+            if constexpr (TAPE) {  // the tile's inputs for the adjoint (fd_tape_row)
                 using V = typename Vec<T>::type;
                 constexpr int W = Vec<T>::W;
                 constexpr int TR = fd_tape_row<T>(R);
@@ -144,8 +172,12 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
 #pragma unroll
                     for (int q2 = 0; q2 < W; ++q2) {
                         const int q = vv * W + q2;
-                        tp[q2] = q < R ? v[q < R ? q : 0] : (q == R ? kb_prev : (q == R + 1 ? kb : (q == R + 2 ? m : T(0))));
-                        if (q == R + 3) tp[q2] = exponent_as<T>(kRescale ? ea : 0);
+                        if (q < R) tp[q2] = v[q < R ? q : 0];
+                        else if (q == R) tp[q2] = kb_prev;
+                        else if (q <= R + C) tp[q2] = kb[q <= R + C ? q - R - 1 : 0];
+                        else if (q == R + C + 1) tp[q2] = m;
+                        else if (q == R + C + 2) tp[q2] = exponent_as<T>(kRescale ? ea : 0);
+                        else tp[q2] = T(0);
                     }
                     __stcs(dst + vv * 32 + lane, t);
                 }
@@ -154,47 +186,62 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
             if constexpr (ORDER == 3) a1 = a1 / (T(1) - m * T(0.25));
             T m2 = T(0);                                 // (1 - beta) = alpha - 1 - m/2 (ORDER 2)
             if constexpr (ORDER == 2) m2 = m * m * T(1.0 / 12.0);
-            T k00 = kb_prev, k01 = kb;                   // k(I, J), k(I, J+1) for I = gR + r
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const T k10 = k00 + v[r];                // k(I+1, J)
-                const T sum = k10 + k01;
-                T d2 = a1 * sum;
-                if constexpr (ORDER == 2) d2 = fma(m2, sum + k00, d2);
-                v[r] += d2;
-                const T k11 = k01 + v[r];                // k(I+1, J+1)
-                k00 = k10;
-                k01 = k11;
-            }
-            kb_prev = kb;
-            top = k01;
-            if (g == groups - 1 && jj == nJ - 1) {
-                double res = static_cast<double>(top);
-                if (kRescale) res = ldexp(res, ea);
-                if (!isfinite(res)) record_error(SK_ERR_NONFINITE);
-                write_result(L, item, P, res);
-                if (TAPE && L.tape_ek != nullptr) {  // exponent of k_hat for the adjoint's scaling
-                    int e2 = 0;
-                    const double t0 = static_cast<double>(top);
-                    if (t0 != 0.0) frexp(t0, &e2);
-                    L.tape_ek[item] = (kRescale ? ea : 0) + e2;
-                }
-            }
-            if (kRescale) {
-                const float mag = fmaxf(fabsf(static_cast<float>(kb_prev)), fabsf(static_cast<float>(top)));
+            // keeps the tile's values within [2^-64, 2^64] after column c: everything the lane
+            // holds or has still to read of this tile moves to the new exponent
+            auto rescale = [&](int c) {
+                const float mag = fmaxf(fabsf(static_cast<float>(kb[c])), fabsf(static_cast<float>(top[c])));
                 if (mag > 0x1p64f || (mag < 0x1p-64f && mag > 0.f)) {
                     const int sh = mag > 0x1p64f ? -64 : 64;
                     const T f = fd_pow2<T>(sh);
 #pragma unroll
                     for (int r = 0; r < R; ++r) v[r] *= f;
-                    kb_prev *= f;
-                    top *= f;
+#pragma unroll
+                    for (int q = 0; q < C; ++q) {
+                        kb[q] *= f;
+                        if (q <= c) top[q] *= f;
+                    }
                     ea -= sh;
                 }
+            };
+            bool wild = false;
+            if constexpr (kRescale && C > 1) wild = !(fabsf(static_cast<float>(m)) <= kFdTileM);
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                T k00 = c == 0 ? kb_prev : kb[c > 0 ? c - 1 : 0], k01 = kb[c];  // k(I, J), k(I, J+1) for I = gR + r
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const T k10 = k00 + v[r];                // k(I+1, J)
+                    const T sum = k10 + k01;
+                    T d2 = a1 * sum;
+                    if constexpr (ORDER == 2) d2 = fma(m2, sum + k00, d2);
+                    v[r] += d2;
+                    const T k11 = k01 + v[r];                // k(I+1, J+1)
+                    k00 = k10;
+                    k01 = k11;
+                }
+                top[c] = k01;
+                if constexpr (kRescale && C > 1) {
+                    if (c + 1 < C && wild) rescale(c);
+                }
             }
+            if (g == groups - 1 && jj == nJ - 1) {
+                double res = static_cast<double>(top[C - 1]);
+                if (kRescale) res = ldexp(res, ea);
+                if (!isfinite(res)) record_error(SK_ERR_NONFINITE);
+                write_result(L, item, P, res);
+                if (TAPE && L.tape_ek != nullptr) {  // exponent of k_hat for the adjoint's scaling
+                    int e2 = 0;
+                    const double t0 = static_cast<double>(top[C - 1]);
+                    if (t0 != 0.0) frexp(t0, &e2);
+                    L.tape_ek[item] = (kRescale ? ea : 0) + e2;
+                }
+            }
+            if (kRescale) rescale(C - 1);
+            kb_prev = kb[C - 1];
             eo = ea;
             if (lane == 31 && gs + 1 < nstrips) {
-                hbuf[jj] = top;
+#pragma unroll
+                for (int c = 0; c < C; ++c) hbuf[jj * C + c] = top[c];
                 if (kRescale) ebuf[jj] = eo;
                 if constexpr (CW > 1) publish_progress(prog + w, gs * nJ + jj + 1);
             }
