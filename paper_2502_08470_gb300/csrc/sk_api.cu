@@ -14,6 +14,8 @@
 #include <utility>
 
 #include "sk_bwd_poly.cuh"
+#include "sk_chain.cuh"
+#include "sk_fwd_chain.cuh"
 #include "sk_common.cuh"
 #include "sk_dispatch.h"
 
@@ -155,8 +157,161 @@ __global__ void sched_scatter_kernel(Launch L, unsigned int* cursor, int32_t* or
 }
 
 // ------------------------------------------------------------------------------------------
+// Tickets and buffers of a strip chain (sk_chain.cuh).  An item without cells gets one ticket.
+// ------------------------------------------------------------------------------------------
+struct ChainBuild {
+    int units;                   // 16-byte units of a hand-off column
+    int ring;                    // buffers an item uses in turn at most
+    int nb;                      // buckets of remaining steps per group
+    int groups;                  // 1: every item's buffers fit together
+    int64_t half;                // units of a group's half of the buffers (groups > 1)
+    unsigned long long* used;    // units taken (groups == 1)
+    unsigned int* total;         // tickets
+    unsigned int* gsize;         // [groups] tickets
+    unsigned int* hist;          // [groups * nb], then the buckets' cursors
+    int64_t* base;               // [items]
+    int32_t* group;              // [items]
+    int4* tickets;
+};
+
+__device__ __forceinline__ void chain_shape(const Launch& L, int64_t item, int& strips, int& cols) {
+    const PairDesc P = decode_pair(L, item);
+    strips = 1;
+    cols = 0;
+    if (P.lx <= 0 || P.ly <= 0) return;
+    strips = static_cast<int>(((P.lx << L.lam) + 31) >> 5);
+    cols = static_cast<int>(P.ly << L.lam);
+}
+__device__ __forceinline__ int64_t chain_need(const ChainBuild& B, int strips, int cols) {
+    return static_cast<int64_t>(min(strips - 1, B.ring)) * ((cols + 7) / 8 * 8) * B.units;
+}
+// Bucket of a strip: kChainLag steps of remaining work each, most first.
+__device__ __forceinline__ int chain_bucket(const ChainBuild& B, int strips, int cols, int s) {
+    const int k = (strips - s) + cols / kChainLag;
+    return B.nb - 1 - min(k, B.nb - 1);
+}
+
+__global__ void chain_base_kernel(Launch L, ChainBuild B) {
+    for (int64_t it = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; it < L.npairs;
+         it += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        int strips, cols;
+        chain_shape(L, it, strips, cols);
+        B.base[it] = static_cast<int64_t>(atomicAdd(B.used, static_cast<unsigned long long>(chain_need(B, strips, cols))));
+        B.group[it] = 0;
+    }
+}
+
+// Groups in the order of L.order (largest first): an item that does not fit the rest of its group's
+// half opens the next group.  One block.
+__global__ void chain_group_kernel(Launch L, ChainBuild B) {
+    __shared__ int64_t need[1024], at[1024];
+    __shared__ int grp[1024];
+    int64_t run = 0;  // thread 0 only
+    int g = 0;
+    for (int64_t k0 = 0; k0 < L.npairs; k0 += 1024) {
+        const int64_t k = k0 + threadIdx.x;
+        const int64_t item = k < L.npairs ? (L.order ? static_cast<int64_t>(L.order[k]) : k) : -1;
+        int strips = 1, cols = 0;
+        if (item >= 0) chain_shape(L, item, strips, cols);
+        need[threadIdx.x] = chain_need(B, strips, cols);
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int q = 0; q < 1024 && k0 + q < L.npairs; ++q) {
+                if (run + need[q] > B.half) {
+                    ++g;
+                    run = 0;
+                }
+                at[q] = run + (g & 1) * B.half;
+                grp[q] = g;
+                run += need[q];
+            }
+        __syncthreads();
+        if (item >= 0) {
+            B.base[item] = at[threadIdx.x];
+            B.group[item] = grp[threadIdx.x];
+        }
+        __syncthreads();
+    }
+}
+
+// One warp per item: lanes take its strips.
+__global__ void chain_hist_kernel(Launch L, ChainBuild B) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
+    for (int64_t it = blockIdx.x * static_cast<int64_t>(blockDim.x >> 5) + (threadIdx.x >> 5); it < L.npairs; it += warps) {
+        int strips, cols;
+        chain_shape(L, it, strips, cols);
+        const int g = B.group[it];
+        for (int s = lane; s < strips; s += 32) atomicAdd(&B.hist[g * B.nb + chain_bucket(B, strips, cols, s)], 1u);
+        if (lane == 0) atomicAdd(&B.gsize[g], static_cast<unsigned int>(strips));
+    }
+}
+
+// Starts of the buckets (in place of hist) and the number of tickets.  One block of 1024.
+__global__ void chain_scan_kernel(ChainBuild B) {
+    __shared__ unsigned int part[1024];
+    const int n = B.groups * B.nb;
+    const int per = (n + 1023) / 1024;
+    const int i0 = threadIdx.x * per, i1 = min(n, i0 + per);
+    unsigned int sum = 0;
+    for (int i = i0; i < i1; ++i) sum += B.hist[i];
+    part[threadIdx.x] = sum;
+    __syncthreads();
+    for (int w = 1; w < 1024; w <<= 1) {
+        const unsigned int v = static_cast<int>(threadIdx.x) >= w ? part[threadIdx.x - w] : 0u;
+        __syncthreads();
+        part[threadIdx.x] += v;
+        __syncthreads();
+    }
+    unsigned int at = part[threadIdx.x] - sum;
+    for (int i = i0; i < i1; ++i) {
+        const unsigned int c = B.hist[i];
+        B.hist[i] = at;
+        at += c;
+    }
+    if (threadIdx.x == 1023) *B.total = part[1023];
+}
+
+__global__ void chain_scatter_kernel(Launch L, ChainBuild B) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
+    for (int64_t it = blockIdx.x * static_cast<int64_t>(blockDim.x >> 5) + (threadIdx.x >> 5); it < L.npairs; it += warps) {
+        int strips, cols;
+        chain_shape(L, it, strips, cols);
+        const int g = B.group[it];
+        unsigned int before = 0;  // ticket + 1 of the strip before the first of these 32
+        for (int s0 = 0; s0 < strips; s0 += 32) {
+            const int s = s0 + lane;
+            unsigned int pos = 0;
+            if (s < strips) pos = atomicAdd(&B.hist[g * B.nb + chain_bucket(B, strips, cols, s)], 1u);
+            unsigned int pred = __shfl_up_sync(kFull, pos, 1) + 1u;
+            if (lane == 0) pred = before;
+            if (s < strips) B.tickets[pos] = make_int4(static_cast<int>(it), s, static_cast<int>(pred), g);
+            before = __shfl_sync(kFull, pos, 31) + 1u;
+        }
+    }
+}
+
+// Clears the units in use (every unit with more than one group).
+__global__ void chain_clear_kernel(uint4* hand, const unsigned long long* used, int64_t all) {
+    const int64_t n = used ? static_cast<int64_t>(*used) : all;
+    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
+         i += static_cast<int64_t>(gridDim.x) * blockDim.x)
+        hand[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// ------------------------------------------------------------------------------------------
 // Argument checks and workspace planning.
 // ------------------------------------------------------------------------------------------
+// Strip chain of a launch (sk_chain.cuh).
+struct ChainPlan {
+    bool on;
+    int units, ring, nb, groups;
+    int64_t cap;      // tickets at most
+    int64_t all;      // 16-byte units of the hand-off buffers
+    size_t off_counts, counts_bytes, off_base, off_group, off_tickets, off_hand;
+};
+
 struct Plan {
     int T;               // 0 = FP64, 1 = FP32 compute
     int nvec, dpad;
@@ -168,8 +323,7 @@ struct Plan {
     int blocks;          // persistent grid
     bool coop;           // cooperative-block kernel (strip pipeline for long pairs)
     int coop_min_strips; // strips from which a pair is swept by a whole block
-    int grid_bpp;        // grid strip pipeline: blocks sharing each pair (0 = off)
-    size_t off_gprog;    // its progress words [npairs][grid_bpp x kCoopWarps]
+    ChainPlan chain;     // polynomial schemes: a warp per strip instead of one per pair
     bool mtile;          // tiled M (wide increments, polynomial schemes)
     int64_t mtile_cols;  // columns of one warp's M strip buffer
     int64_t mtile_off;   // byte offset of that buffer in a warp slot
@@ -190,10 +344,54 @@ struct Plan {
 
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
-constexpr int kGridMinBlocks = 8;  // fewest blocks a pair's ring may span in the grid strip pipeline
 // Bytes of precomputed M a forward holds at once (the chunk of items whose M the tensor cores
 // wrote before the chunk's sweep); a chunk is a whole number of the sweep's resident warps.
 constexpr size_t kMxBudget = size_t(8) << 30;
+// Bytes of hand-off buffers a strip chain may take, the fewest buffers a pair with more strips may
+// use in turn, and the most buckets its tickets are sorted into.  8 GB holds every buffer of 4096
+// uneven pairs of 64 .. 4096 points (7.7 GB at N = 6 in FP32).
+constexpr size_t kChainBudget = size_t(8) << 30;
+constexpr int64_t kChainMinRing = 64;
+constexpr int64_t kChainMaxBuckets = 1 << 16;
+
+// Plans a chain over npairs items of at most `strips` strips and `cols` columns, its workspace from
+// offset `off` (advanced past it); false when the shape does not suit one.  limit: bytes available
+// for the hand-off buffers.
+bool plan_chain(ChainPlan& c, size_t& off, int64_t npairs, int64_t strips, int64_t cols, int units, size_t limit) {
+    c = ChainPlan{};
+    c.units = units;
+    c.cap = npairs * strips;
+    if (npairs <= 0 || strips < 2 || c.cap > (int64_t(1) << 26)) return false;
+    const int64_t stride = (cols + 7) / 8 * 8 * units;  // whole batches of up to 8 columns
+    const int64_t budget = static_cast<int64_t>(std::min(limit, kChainBudget) / 16);
+    int64_t ring = strips - 1;
+    const int64_t room = npairs > 1 ? budget / 2 : budget;  // a pair's buffers lie in one half
+    if (ring * stride > room) ring = room / stride;
+    if (ring < std::min(strips - 1, kChainMinRing)) return false;
+    const int64_t bound = npairs * ring * stride;
+    c.ring = static_cast<int>(ring);
+    // greedy groups are at least half full
+    const int64_t groups = bound <= budget ? 1 : 2 * (bound / (budget / 2)) + 2;
+    const int64_t nb = strips + cols / kChainLag + 1;
+    if (nb * groups > kChainMaxBuckets) return false;
+    c.nb = static_cast<int>(nb);
+    c.groups = static_cast<int>(groups);
+    c.all = groups > 1 ? budget / 2 * 2 : bound;
+    // cleared before each launch: used, total, gsize and gdone, strips done per item, histogram
+    c.off_counts = off;
+    c.counts_bytes = align256(16 + (2 * static_cast<size_t>(groups) + static_cast<size_t>(npairs) + static_cast<size_t>(nb * groups)) * 4);
+    off += c.counts_bytes;
+    c.off_base = off;
+    off += align256(static_cast<size_t>(npairs) * 8);
+    c.off_group = off;
+    off += align256(static_cast<size_t>(npairs) * 4);
+    c.off_tickets = off;
+    off += align256(static_cast<size_t>(c.cap) * sizeof(int4));
+    c.off_hand = off;
+    off += align256(static_cast<size_t>(c.all) * 16);
+    c.on = true;
+    return true;
+}
 
 int check_paths(const sk_paths* P, const char* name, int d) {
     if (!P) return fail(SK_ERR_INVALID_ARG, "%s is NULL", name);
@@ -259,11 +457,32 @@ int check_options(const sk_options* o, int32_t d, int32_t dtype) {
     return SK_OK;
 }
 
+// Whether to give every strip of a pair a warp of its own rather than every pair one, estimated in
+// warp steps.  One warp per pair takes as long as the longest pair or as the whole batch at full
+// rate, whichever is more; a chain takes its fill (a strip starts kChainLag steps after the one
+// below it) or the whole batch, with a tenth more instructions a step for the hand-off.  Half the
+// resident warps reach the full FP32 rate, a quarter the FP64 rate.  The batch's total is taken from
+// the mean path lengths, which is all that the host knows.
+bool chain_pays(const sk_paths* X, const sk_paths* Y, int64_t points, int lam, int64_t npairs, int64_t strips,
+                int64_t cols, int64_t resident, int T) {
+    if (X->count <= 0 || Y->count <= 0) return false;
+    const double rx = std::max(1.0, static_cast<double>(X->rows_total) / X->count - points) * (1 << lam);
+    const double ry = std::max(1.0, static_cast<double>(Y->rows_total) / Y->count - points) * (1 << lam);
+    const double total = static_cast<double>(npairs) * std::ceil(rx / 32.0) * std::max(ry, 32.0);
+    const double full = total / (static_cast<double>(resident) / (T ? 2 : 4));
+    const double one = std::max(static_cast<double>(strips) * std::max<int64_t>(cols, 32), full);
+    const double chained = std::max(static_cast<double>(cols + kChainLag * strips), 1.1 * full);
+    return chained < 0.9 * one;
+}
+
 // allow_coop: the caller launches p.kern itself with p.threads (the plain forward); adjoint
 // plans reuse this layout with their own one-warp-per-pair kernels and pass false.  tape: the
 // forward records a tape (one warp per pair; its own kernels for the approximation scheme).
+// chain_limit: bytes a strip chain's buffers may take (0: no chain).
+constexpr size_t kChainAny = ~size_t(0);
 int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, const sk_options* o,
-                 int mode, int64_t npairs, Plan& p, bool allow_coop = false, bool tape = false) {
+                 int mode, int64_t npairs, Plan& p, bool allow_coop = false, bool tape = false,
+                 size_t chain_limit = kChainAny) {
     int rc;
     if ((rc = check_options(o, d, dtype)) != SK_OK) return rc;
     if ((rc = check_paths(X, "X", d)) != SK_OK) return rc;
@@ -293,8 +512,8 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     // instead (produce_m_strip).
     const bool mt_eligible = poly && p.T == 1 && p.dpad >= 12;
     p.mtile = mt_eligible && !(o->flags & SK_FLAG_NO_TILED_M);
-    auto kernel_for = [&](bool coop) -> const void* {
-        return poly ? fwd_poly_kernel_ptr(p.T, o->scheme == SK_POLY_INTERP, o->degree, coop, p.mtile, tape)
+    auto kernel_for = [&](bool coop) -> const void* {  // coop: the FD schemes' pipelined blocks
+        return poly ? fwd_poly_kernel_ptr(p.T, o->scheme == SK_POLY_INTERP, o->degree, false, p.mtile, tape)
                     : fwd_fd_kernel_ptr(p.T, o->scheme == SK_FD2 ? 2 : o->scheme == SK_FD_IMPLICIT ? 3 : 1, lam, coop, tape);
     };
     p.kern = kernel_for(false);
@@ -329,10 +548,14 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     p.threads = (wpb_req ? wpb_req : kFwdWarps) * 32;
     p.coop = false;
     p.coop_min_strips = 0;
-    p.grid_bpp = 0;
+    p.chain = ChainPlan{};
     const int esize = p.T ? 4 : 8;
     p.smem_x = 0;
-    auto xsmem = [&](int threads) { return p.mtile ? (threads / 32) * 32 * p.dpad * esize : 0; };
+    // shared memory: the x rows of tiled M; a chained strip's x rows and M in FP32
+    auto xsmem = [&](int threads) -> int {
+        if (p.chain.on) return p.T ? (threads / 32) * chain_smem_floats(p.dpad) * 4 : 0;
+        return p.mtile ? (threads / 32) * 32 * p.dpad * esize : 0;
+    };
     auto occupancy = [&](const void* k, int threads, int* per) -> int {
         const int sm = xsmem(threads);
         if (sm > 48 * 1024) SK_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
@@ -342,48 +565,38 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     SK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     if ((rc = occupancy(p.kern, p.threads, &per_sm)) != SK_OK) return rc;
     if (per_sm < 1) per_sm = 1;
-    // Strip pipeline: a pair of many strips swept by one warp is a serial chain of
-    // nstrips x cols steps; when the batch cannot fill the GPU with one warp per pair, long pairs
-    // are swept by blocks of kCoopWarps warps instead (one strip per warp, pipelined).
-    if (allow_coop && pipe_req >= 0) {
-        const int rows_per_lane = poly ? 1 : (lam < 4 ? (1 << lam) : 16);
-        // rows of the longest X path: its increments (one fewer than its points in points mode)
-        const int64_t max_rows = std::max<int64_t>(X->max_len - ((o->flags & SK_FLAG_INCREMENTS) ? 0 : 1), 1) << lam;
+    // A pair of many strips swept by one warp is a serial chain of nstrips x cols steps.  When the
+    // batch cannot fill the GPU with one warp per pair, the strips are spread over several warps:
+    // the polynomial schemes give every strip a warp of its own (strip chain, below), the FD schemes
+    // sweep a pair with a block of kCoopWarps warps.
+    const int64_t points = (o->flags & SK_FLAG_INCREMENTS) ? 0 : 1;
+    // rows and columns of the longest paths: their increments (one fewer than their points)
+    const int64_t max_rows = std::max<int64_t>(X->max_len - points, 1) << lam;
+    const int64_t max_cols = std::max<int64_t>(Y->max_len - points, 1) << lam;
+    if (allow_coop && pipe_req >= 0 && !poly) {
+        const int rows_per_lane = lam < 4 ? (1 << lam) : 16;
         const int64_t max_strips = ((max_rows / rows_per_lane) + 31) / 32;
         const bool forced = pipe_req > 0;
         const int64_t resident = static_cast<int64_t>(sms) * per_sm * (p.threads / 32);
         if (max_strips >= 2 && (forced || (max_strips >= 2 * kCoopWarps && npairs < 4 * resident))) {
-            // Pipelined warps are all on the pipeline's critical path, so a strip's tiled-M build
-            // delays the whole chain: per-cell M measured faster there (4096 pairs of 64..4096-point
-            // paths, d = 16: 101 against 118 ms).
-            const bool mt_one = p.mtile;
-            p.mtile = false;
             const void* ck = kernel_for(true);
             int cper = 0;
             if (ck && (rc = occupancy(ck, kCoopWarps * 32, &cper)) != SK_OK) return rc;
-            if (!(ck && cper >= 1)) p.mtile = mt_one;
             if (ck && cper >= 1) {
                 p.kern = ck;
                 p.coop = true;
-                // once a batch is pipelined at all, every pair of two or more strips is (measured on
-                // 4096 pairs of 64..4096-point paths: 101 ms against 197 ms with only pairs of
-                // 2 kCoopWarps strips or more)
+                // once a batch is pipelined at all, every pair of two or more strips is
                 p.coop_min_strips = 2;
                 p.threads = kCoopWarps * 32;
                 per_sm = cper;
-                // Few long pairs: one block per pair would leave SMs idle, so each pair's ring of
-                // warps spans several co-resident blocks (no more than its strips can use).  A
-                // step costs several times more there (GPU-scope hand-off), so the ring must
-                // spread over at least kGridMinBlocks blocks: 1 pair of 16385-point paths ran
-                // 5.5x faster, 8 pairs of 4097 points 1.4x, but 32 pairs of 2049 points (4 blocks
-                // each) 1.6x slower and 64 pairs of 1025 points (2 each) 2.8x slower.
-                const int64_t rblocks = static_cast<int64_t>(sms) * cper;
-                if (poly && npairs > 0 && max_strips >= kGridMinBlocks * kCoopWarps) {
-                    const int64_t bpp = std::min<int64_t>(rblocks / npairs, (max_strips + kCoopWarps - 1) / kCoopWarps);
-                    if (bpp >= kGridMinBlocks) p.grid_bpp = static_cast<int>(bpp);
-                }
             }
         }
+    }
+    bool want_chain = false;
+    const int64_t strips = (max_rows + 31) / 32;
+    if (poly && chain_limit > 0 && pipe_req >= 0 && wpb_req == 0 && strips >= 2 && npairs > 0) {
+        want_chain = pipe_req > 0 || chain_pays(X, Y, points, lam, npairs, strips, max_cols,
+                                                static_cast<int64_t>(sms) * per_sm * kFwdWarps, p.T);
     }
     // Tensor-core M: in place of the per-cell or tiled M, the FP32 approximation scheme's
     // one-warp-per-pair sweep reads each cell's M from a buffer that a tcgen05 GEMM fills per chunk
@@ -399,16 +612,30 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     p.mx_stride = 0;
     p.mx_chunk = npairs;
     const bool mt_chosen = p.mtile;
-    if (p.T == 1 && o->scheme == SK_POLY_APPROX && p.dpad >= 8 && p.dpad <= 32 && !p.coop &&
-        !(o->flags & SK_FLAG_NO_TC)) {
+    // groups of four warp steps, 32 lanes x float4 each
+    const int64_t mx_steps = (strips - 1) * std::max<int64_t>(max_cols, 32) + 31 + max_cols;
+    const int64_t mx_bytes = static_cast<int64_t>(align256(static_cast<size_t>((mx_steps + 3) / 4) * 32 * 16));
+    const bool mx_scheme = p.T == 1 && o->scheme == SK_POLY_APPROX && p.dpad >= 8 && p.dpad <= 32 && !(o->flags & SK_FLAG_NO_TC);
+    const int chain_u = p.T ? chain_units<float>(o->degree) : chain_units<double>(o->degree);
+    if (want_chain) {
+        const void* ck = fwd_poly_kernel_ptr(p.T, o->scheme == SK_POLY_INTERP, o->degree, true, false, tape);
+        size_t none = 0;
+        if (ck && plan_chain(p.chain, none, npairs, strips, max_cols, chain_u, chain_limit)) {
+            int cper = 0;
+            if ((rc = occupancy(ck, kFwdWarps * 32, &cper)) != SK_OK) return rc;  // with the chain's x rows
+            p.chain.on = cper >= 1;
+            if (p.chain.on) {
+                p.kern = ck;
+                p.threads = kFwdWarps * 32;
+                p.mtile = false;
+                per_sm = cper;
+            }
+        }
+    }
+    if (!p.chain.on && mx_scheme) {
         const void* km = fwd_poly_kernel_ptr(p.T, false, o->degree, false, false, tape, true);
         if (km) {
-            const int64_t pts = (o->flags & SK_FLAG_INCREMENTS) ? 0 : 1;
-            const int64_t rmax = std::max<int64_t>(X->max_len - pts, 1) << lam;
-            const int64_t cmax = std::max<int64_t>(Y->max_len - pts, 1) << lam;
-            const int64_t nsteps = ((rmax + 31) / 32 - 1) * std::max<int64_t>(cmax, 32) + 31 + cmax;
-            // groups of four warp steps, 32 lanes x float4 each
-            const int64_t stride = static_cast<int64_t>(align256(static_cast<size_t>((nsteps + 3) / 4) * 32 * 16));
+            const int64_t stride = mx_bytes;
             int mper = 0;
             p.mtile = false;  // no x-row staging for this kernel
             if ((rc = occupancy(km, p.threads, &mper)) != SK_OK) return rc;
@@ -433,7 +660,7 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
         }
     }
     const int wpb = p.threads / 32;
-    int64_t want = p.coop ? (p.grid_bpp > 0 ? npairs * p.grid_bpp : npairs) : (npairs + wpb - 1) / wpb;
+    int64_t want = p.coop ? npairs : ((p.chain.on ? p.chain.cap : npairs) + wpb - 1) / wpb;
     int64_t cap = static_cast<int64_t>(sms) * per_sm;
     p.blocks = static_cast<int>(want < cap ? (want > 0 ? want : 1) : cap);
     p.buf_cols = (Y->max_len << lam) + 1;
@@ -442,6 +669,7 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     p.mtile_cols = std::max<int64_t>(Y->max_len << lam, 1);
     p.mtile_off = p.slot_bytes;
     if (p.mtile) p.slot_bytes += static_cast<int64_t>(align256(static_cast<size_t>(2 * 32 * p.mtile_cols * esize)));
+    if (p.chain.on) p.slot_bytes = 0;  // a chained warp hands on through the chain's buffers
 
     size_t off = 0;
     p.off_incx = off;
@@ -456,8 +684,10 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     off += align256(static_cast<size_t>(npairs) * sizeof(int32_t));
     p.off_scratch = off;
     off += static_cast<size_t>(p.blocks) * wpb * static_cast<size_t>(p.slot_bytes);
-    p.off_gprog = off;
-    if (p.grid_bpp > 0) off += align256(static_cast<size_t>(p.blocks) * wpb * sizeof(int));
+    if (p.chain.on) {
+        off = align256(off);
+        plan_chain(p.chain, off, npairs, strips, max_cols, chain_u, chain_limit);
+    }
     p.off_xt = p.off_yt = p.off_mx = off;
     if (p.mx) {
         p.off_xt = off;
@@ -537,11 +767,79 @@ int plan_tape(const sk_paths* X, const sk_paths* Y, const sk_options* o, int T, 
     return SK_OK;
 }
 
+// The plan of a forward call whose workspace holds `bytes`.  Where a chain does not fit, it gets fewer
+// buffers, or every pair one warp: a workspace that was large enough without a chain stays so.
+int plan_forward_within(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, const sk_options* o, int mode,
+                        int64_t npairs, Plan& p, bool tape, size_t bytes) {
+    int rc = plan_forward(X, Y, d, dtype, o, mode, npairs, p, !tape, tape);
+    if (rc != SK_OK || p.total <= bytes || !p.chain.on) return rc;
+    const size_t rest = p.total - align256(static_cast<size_t>(p.chain.all) * 16);
+    if ((rc = plan_forward(X, Y, d, dtype, o, mode, npairs, p, !tape, tape, bytes > rest ? bytes - rest : 0)) != SK_OK) return rc;
+    if (p.total <= bytes || !p.chain.on) return rc;
+    return plan_forward(X, Y, d, dtype, o, mode, npairs, p, !tape, tape, 0);
+}
+
+// Fills a launch's chain fields: clears the hand-off buffers and writes the tickets (stream-ordered;
+// `order` and `hist` are the workspace of the counting sort, its queue and histogram clear).
+int launch_chain_tickets(const ChainPlan& c, Launch& L, bool sorted, char* base, size_t off_hist, size_t off_order,
+                         cudaStream_t st) {
+    char* counts = base + c.off_counts;
+    ChainBuild B;
+    B.units = c.units;
+    B.ring = c.ring;
+    B.nb = c.nb;
+    B.groups = c.groups;
+    B.half = c.all / 2;
+    B.used = reinterpret_cast<unsigned long long*>(counts);
+    B.total = reinterpret_cast<unsigned int*>(counts + 8);
+    B.gsize = reinterpret_cast<unsigned int*>(counts + 16);
+    unsigned int* gdone = B.gsize + c.groups;
+    int* done = reinterpret_cast<int*>(gdone + c.groups);
+    B.hist = reinterpret_cast<unsigned int*>(done + L.npairs);
+    B.base = reinterpret_cast<int64_t*>(base + c.off_base);
+    B.group = reinterpret_cast<int32_t*>(base + c.off_group);
+    B.tickets = reinterpret_cast<int4*>(base + c.off_tickets);
+    L.ch_tickets = B.tickets;
+    L.ch_total = B.total;
+    L.ch_hand = reinterpret_cast<ChainUnit*>(base + c.off_hand);
+    L.ch_base = B.base;
+    L.ch_ring = c.ring;
+    L.ch_groups = c.groups;
+    L.ch_done = done;
+    L.ch_gsize = B.gsize;
+    L.ch_gdone = gdone;
+    L.order = nullptr;
+    SK_CUDA(cudaMemsetAsync(counts, 0, c.counts_bytes, st));
+    const int sb = static_cast<int>(std::min<int64_t>((L.npairs + 255) / 256, 4096));
+    const int wb = static_cast<int>(std::min<int64_t>((L.npairs + 7) / 8, 4096));
+    if (c.groups == 1) {
+        chain_base_kernel<<<sb, 256, 0, st>>>(L, B);
+    } else {
+        Launch S = L;
+        if (sorted && L.npairs > 1) {  // largest first
+            unsigned int* hist = reinterpret_cast<unsigned int*>(base + off_hist);
+            int32_t* order = reinterpret_cast<int32_t*>(base + off_order);
+            sched_hist_kernel<<<sb, 256, 0, st>>>(L, hist);
+            sched_scan_kernel<<<1, 32, 0, st>>>(hist, hist + 65);
+            sched_scatter_kernel<<<sb, 256, 0, st>>>(L, hist + 65, order);
+            S.order = order;
+        }
+        chain_group_kernel<<<1, 1024, 0, st>>>(S, B);
+    }
+    chain_hist_kernel<<<wb, 256, 0, st>>>(L, B);
+    chain_scan_kernel<<<1, 1024, 0, st>>>(B);
+    chain_scatter_kernel<<<wb, 256, 0, st>>>(L, B);
+    const int cb = static_cast<int>(std::min<int64_t>((c.all + 255) / 256, 4096));
+    chain_clear_kernel<<<cb, 256, 0, st>>>(reinterpret_cast<uint4*>(base + c.off_hand), c.groups == 1 ? B.used : nullptr, c.all);
+    SK_CUDA(cudaGetLastError());
+    return SK_OK;
+}
+
 int run_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, const sk_options* o, int mode,
                 const int64_t* pa, const int64_t* pb, int64_t npairs, double* out, int64_t ldo, void* ws,
                 size_t ws_bytes, void* stream, void* tape = nullptr, size_t tape_bytes = 0, int64_t item_base = 0) {
     Plan p;
-    int rc = plan_forward(X, Y, d, dtype, o, mode, npairs, p, tape == nullptr, tape != nullptr);
+    int rc = plan_forward_within(X, Y, d, dtype, o, mode, npairs, p, tape != nullptr, ws ? ws_bytes : kChainAny);
     if (rc != SK_OK) return rc;
     TapePlan tp{0, 0, 0, 0};
     if (tape) {
@@ -594,9 +892,6 @@ int run_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, 
     L.tape_stride = static_cast<int64_t>(tp.stride);
     L.tape_ek = tape ? static_cast<int*>(tape) : nullptr;
     L.coop_min_strips = p.coop_min_strips;
-    L.grid_bpp = p.grid_bpp;
-    L.gprog = p.grid_bpp > 0 ? reinterpret_cast<int*>(base + p.off_gprog) : nullptr;
-    if (p.grid_bpp > 0) SK_CUDA(cudaMemsetAsync(L.gprog, 0, static_cast<size_t>(p.blocks) * (p.threads / 32) * sizeof(int), st));
     L.mtile = p.mtile ? 1 : 0;
     L.mtile_cols = static_cast<int32_t>(p.mtile_cols);
     L.mtile_off = p.mtile_off;
@@ -643,7 +938,9 @@ int run_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, 
             }
         }
         SK_CUDA(cudaMemsetAsync(base + p.off_queue, 0, 256 + align256(2 * 65 * sizeof(unsigned int)), st));
-        if (!(o->flags & SK_FLAG_NO_SORT) && n > 1) {
+        if (p.chain.on) {
+            if ((rc = launch_chain_tickets(p.chain, C, !(o->flags & SK_FLAG_NO_SORT), base, p.off_hist, p.off_order, st)) != SK_OK) return rc;
+        } else if (!(o->flags & SK_FLAG_NO_SORT) && n > 1) {
             unsigned int* hist = reinterpret_cast<unsigned int*>(base + p.off_hist);
             int32_t* order = reinterpret_cast<int32_t*>(base + p.off_order);
             int sb = static_cast<int>((n + 255) / 256);
@@ -659,24 +956,9 @@ int run_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, 
             SK_CUDA(launch_m_tc(p.kp, C, base + p.off_xt, base + p.off_yt, p.xt_nblk, p.yt_nblk,
                                 reinterpret_cast<float*>(base + p.off_mx), p.mx_stride, sms, st));
         void* args[] = {&C, &buf_cols};
-        if (p.grid_bpp > 0) {
-            // the blocks of a pair wait on one another: launch them co-resident
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(p.blocks);
-            cfg.blockDim = dim3(p.threads);
-            cfg.dynamicSmemBytes = static_cast<size_t>(smem);
-            cfg.stream = st;
-            cudaLaunchAttribute attr;
-            attr.id = cudaLaunchAttributeCooperative;
-            attr.val.cooperative = 1;
-            cfg.attrs = &attr;
-            cfg.numAttrs = 1;
-            SK_CUDA(cudaLaunchKernelExC(&cfg, p.kern, args));
-        } else {
-            const int64_t want = p.coop ? n : (n + wpb - 1) / wpb;
-            const int blocks = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(want, p.blocks)));
-            SK_CUDA(cudaLaunchKernel(p.kern, dim3(blocks), dim3(p.threads), args, smem, st));
-        }
+        const int64_t want = p.coop ? n : ((p.chain.on ? p.chain.cap : n) + wpb - 1) / wpb;
+        const int blocks = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(want, p.blocks)));
+        SK_CUDA(cudaLaunchKernel(p.kern, dim3(blocks), dim3(p.threads), args, smem, st));
     }
     if (timed) {
         SK_CUDA(cudaEventRecord(t_ev1, st));
@@ -724,7 +1006,7 @@ struct BwdPlan {
 
 int plan_backward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, const sk_options* o, int mode,
                   int64_t npairs, BwdPlan& b) {
-    int rc = plan_forward(X, Y, d, dtype, o, mode, npairs, b.f);
+    int rc = plan_forward(X, Y, d, dtype, o, mode, npairs, b.f, false, false, 0);
     if (rc != SK_OK) return rc;
     if (o->scheme != SK_POLY_APPROX)
         return fail(SK_ERR_UNSUPPORTED, "sigkernel_backward supports the polynomial approximation scheme");
@@ -901,6 +1183,7 @@ struct TapeBwdPlan {
     Plan f;
     TapePlan t;
     const void* kern;
+    ChainPlan chain;     // a warp per strip instead of one per pair
     const void* ckern;
     int smem_bytes, cblocks, csmem, cC;
     int64_t cols_max, off_rbuf, off_rexp, slot_bytes, mb_stride, acc_bytes;
@@ -913,8 +1196,8 @@ struct TapeBwdPlan {
 };
 
 int plan_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, const sk_options* o, int mode,
-                       int64_t npairs, TapeBwdPlan& b) {
-    int rc = plan_forward(X, Y, d, dtype, o, mode, npairs, b.f);
+                       int64_t npairs, TapeBwdPlan& b, bool chain_ok = true) {
+    int rc = plan_forward(X, Y, d, dtype, o, mode, npairs, b.f, false, false, 0);
     if (rc != SK_OK) return rc;
     const Plan& p = b.f;
     if ((rc = plan_tape(X, Y, o, p.T, npairs, b.t)) != SK_OK) return rc;
@@ -982,7 +1265,28 @@ int plan_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t 
     if (cper_sm < 1) return fail(SK_ERR_UNSUPPORTED, "contraction kernel does not fit an SM");
     b.tc_sms = sms;
     b.cblocks = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(npairs, static_cast<int64_t>(sms) * cper_sm)));
-    const int64_t want = (npairs + kFwdWarps - 1) / kFwdWarps;
+    int64_t want = (npairs + kFwdWarps - 1) / kFwdWarps;
+    // too few pairs to fill the GPU with one warp each: a warp per strip, as in the forward
+    b.chain = ChainPlan{};
+    const void* chain_kern = fd ? nullptr : bwd_chain_ptr(p.T, o->degree, interp);
+    const int64_t points = (o->flags & SK_FLAG_INCREMENTS) ? 0 : 1;
+    const int64_t strips = ((std::max<int64_t>(X->max_len - points, 1) << o->dyadic) + 31) / 32;
+    const int64_t max_cols = std::max<int64_t>(Y->max_len - points, 1) << o->dyadic;
+    const int units = p.T ? chain_units<float>(N) : chain_units<double>(N);
+    if (chain_kern && strips >= 2 && npairs > 0 && chain_ok && !(o->flags & SK_FLAG_NO_STRIP_PIPELINE) &&
+        ((o->flags & SK_FLAG_STRIP_PIPELINE) || chain_pays(X, Y, points, o->dyadic, npairs, strips, max_cols,
+                                                           static_cast<int64_t>(sms) * per_sm * kFwdWarps, p.T))) {
+        int cper = 0;
+        SK_CUDA(cudaFuncSetAttribute(chain_kern, cudaFuncAttributeMaxDynamicSharedMemorySize, b.smem_bytes));
+        SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cper, chain_kern, p.threads, b.smem_bytes));
+        size_t none = 0;
+        if (cper >= 1 && plan_chain(b.chain, none, npairs, strips, max_cols, units, kChainAny)) {
+            b.kern = chain_kern;
+            per_sm = cper;
+            b.slot_bytes = 0;
+            want = (b.chain.cap + kFwdWarps - 1) / kFwdWarps;
+        }
+    }
     b.f.blocks = static_cast<int>(std::max<int64_t>(1, std::min(want, static_cast<int64_t>(sms) * per_sm)));
     size_t o2 = p.off_scratch;
     b.off_gincx = o2;
@@ -992,6 +1296,8 @@ int plan_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t 
     b.off_scratch = o2;
     o2 += static_cast<size_t>(b.f.blocks) * kFwdWarps * static_cast<size_t>(b.slot_bytes);
     o2 = align256(o2);
+    if (b.chain.on)
+        plan_chain(b.chain, o2, npairs, strips, max_cols, units, kChainAny);
     b.off_mbuf = o2;
     o2 += static_cast<size_t>(npairs) * static_cast<size_t>(b.mb_stride);
     o2 = align256(o2);
@@ -1065,11 +1371,12 @@ int launch_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int32_
         SK_CUDA(launch_tc_operands(b.tcN, L.X, inc_mode, clam, p.dpad, b.nrb, base + b.off_xt, st));
         if (!p.same_xy) SK_CUDA(launch_tc_operands(b.tcN, L.Y, inc_mode, clam, p.dpad, b.ncb, base + b.off_yt, st));
     }
-    SK_CUDA(cudaMemsetAsync(base + p.off_queue, 0, 256, st));
-    if (!(o->flags & SK_FLAG_NO_SORT) && npairs > 1) {
+    SK_CUDA(cudaMemsetAsync(base + p.off_queue, 0, 256 + align256(2 * 65 * sizeof(unsigned int)), st));
+    if (b.chain.on) {
+        if ((rc = launch_chain_tickets(b.chain, L, !(o->flags & SK_FLAG_NO_SORT), base, p.off_hist, p.off_order, st)) != SK_OK) return rc;
+    } else if (!(o->flags & SK_FLAG_NO_SORT) && npairs > 1) {
         unsigned int* hist = reinterpret_cast<unsigned int*>(base + p.off_hist);
         int32_t* order = reinterpret_cast<int32_t*>(base + p.off_order);
-        SK_CUDA(cudaMemsetAsync(hist, 0, align256(2 * 65 * sizeof(unsigned int)), st));
         int sb = static_cast<int>(std::min<int64_t>((npairs + 255) / 256, 4096));
         sched_hist_kernel<<<sb, 256, 0, st>>>(L, hist);
         sched_scan_kernel<<<1, 32, 0, st>>>(hist, hist + 65);
@@ -1109,6 +1416,9 @@ int run_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t d
     if (b.f.same_xy && gY && gY != gX)
         return fail(SK_ERR_INVALID_ARG, "X and Y are the same paths: pass grad_Y = NULL or grad_Y = grad_X");
     if (!tape || tape_bytes < b.t.total) return fail(SK_ERR_WORKSPACE, "tape missing or smaller than %zu bytes", b.t.total);
+    if (ws && ws_bytes < b.total && b.chain.on &&  // a workspace without room for a chain's buffers
+        (rc = plan_backward_tape(X, Y, d, dtype, o, mode, npairs, b, false)) != SK_OK)
+        return rc;
     if (npairs == 0) return SK_OK;
     if (!gout) return fail(SK_ERR_INVALID_ARG, "grad_out is NULL");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -1534,6 +1844,17 @@ int run_mmd2_test(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t dtyp
 
 void set_last_error(const char* msg) { t_last_error = msg; }
 
+int pairs_need(const sk_paths* X, const sk_paths* Y, int32_t d, int64_t npairs, const sk_options* opt, size_t capacity,
+               size_t* need) {
+    t_last_error.clear();
+    *need = 0;
+    if (!opt || !X || !Y) return fail(SK_ERR_INVALID_ARG, "NULL argument");
+    Plan p;
+    const int rc = plan_forward_within(X, Y, d, SK_F64, opt, kPairsList, npairs, p, false, capacity);
+    if (rc == SK_OK) *need = p.total;
+    return rc;
+}
+
 }  // namespace sk
 
 using namespace sk;
@@ -1585,7 +1906,7 @@ int sigkernel_autotune(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t 
         sk_options co = cand_options(all[c]);
         Plan p;
         if ((rc = plan_forward(X, Y, d, dtype, &co, mode, n, p, true)) != SK_OK) return rc;
-        if (all[c].pipe > 0 && !p.coop) continue;            // no pair spans two strips
+        if (all[c].pipe > 0 && !p.coop && !p.chain.on) continue;  // no pair spans two strips
         if (all[c].pipe < 0 && all[c].mt > 0 && !p.mtile) continue;  // tiled M not applicable
         cands[ncand++] = all[c];
         ws_bytes = std::max(ws_bytes, p.total);
@@ -1720,7 +2041,14 @@ int sigkernel_workspace_size(int32_t op, const sk_paths* X, const sk_paths* Y, i
         default:
             return fail(SK_ERR_UNSUPPORTED, "workspace for op %d", op);
     }
-    if (rc == SK_OK) *bytes = p.total;
+    if (rc == SK_OK) {
+        *bytes = p.total;
+        // sigkernel_forward_tape takes the same workspace and may plan another route
+        const int mode = op == SK_OP_PAIRS ? kPairsList : (opt->flags & SK_FLAG_SYMMETRIC) ? kGramUpper : kGramFull;
+        Plan pt;
+        if (plan_forward(X, Y, d, dtype, opt, mode, p.npairs, pt, false, true) == SK_OK) *bytes = std::max(*bytes, pt.total);
+        t_last_error.clear();
+    }
     return rc;
 }
 

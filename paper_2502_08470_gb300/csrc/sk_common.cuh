@@ -21,6 +21,9 @@ constexpr int kJF64 = 10;        // ... and in FP64
 constexpr int kMaxRefined = 131072;  // bound on (rows per path) << lambda (keeps step counters in int32)
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kFwdWarps = 4;     // warps per block of the persistent wavefront kernels
+// Warps of a block that sweep one long pair of the FD schemes together (strip pipeline).  Sixteen
+// measured faster than eight on few long pairs and on uneven batches.
+constexpr int kCoopWarps = 16;
 
 // Device error word: the first SK_ERR_* code recorded by any kernel of the library.
 extern __device__ int g_sk_error;
@@ -109,6 +112,8 @@ struct PairDesc {
     int64_t lx, ly;          // increments per path (>= 0), or -1 when the path is invalid
 };
 
+struct ChainUnit;
+
 struct Launch {
     PathSet X, Y;
     int32_t nvec;            // 16-byte chunks per increment row
@@ -132,7 +137,7 @@ struct Launch {
     void* tape;
     int64_t tape_stride;     // bytes per work item
     int* tape_ek;            // [npairs]
-    // Cooperative strip pipeline (kernels launched with several warps per pair): a pair with at
+    // Cooperative strip pipeline (FD kernels launched with several warps per pair): a pair with at
     // least this many strips is swept by all warps of a block together; shorter pairs get one
     // warp each.
     int32_t coop_min_strips;
@@ -146,20 +151,27 @@ struct Launch {
     // Gram modes: work item k of this launch is item k + item_base of the whole Gram (a call can
     // sweep a sub-range of a Gram's items; its tape and queue are indexed by k).
     int64_t item_base;
-    // Grid strip pipeline (few long pairs): when nonzero, grid_bpp blocks of the pipelined kernel
-    // share each work item, all launched co-resident; block b takes slot b / grid_bpp of the queue
-    // order and is part b % grid_bpp of that item's ring of grid_bpp x CW warps.  The ring's
-    // progress words are gprog[slot][grid_bpp x CW] in global memory (zeroed before the launch).
-    int32_t grid_bpp;
-    int* gprog;
     // Polls a strip-pipeline hand-off wait makes before it gives up (0 = kSpinLimit).
     uint32_t wait_limit;
-    // Precomputed M (FP32 approximation scheme, one warp per pair): per work item k of the launch,
+    // Precomputed M (FP32 approximation scheme): per work item k of the launch,
     // at byte offset k * mx_stride, the cells' M_ij / 4^lambda in the warp's schedule, in groups of
     // four warp steps: lane r's M of steps 4G .. 4G + 3 is the float4 at index 32 G + r.  NULL when
     // the cells form M themselves.
     const float* mx;
     int64_t mx_stride;
+    // Strip chain (sk_chain.cuh): the tickets in order, (work item, strip, ticket of the strip before
+    // + 1, group), and how many there are; the hand-off buffers, each item's first unit in them and
+    // the buffers an item uses in turn; strips done per item; and, with more than one group, the
+    // tickets of each and how many are done.  Counters are cleared before the launch.
+    const int4* ch_tickets;
+    const unsigned int* ch_total;
+    ChainUnit* ch_hand;
+    const int64_t* ch_base;
+    int32_t ch_ring;
+    int32_t ch_groups;
+    int* ch_done;
+    const unsigned int* ch_gsize;
+    unsigned int* ch_gdone;
 };
 
 // Width, in elements of T, of one lane's tape row.
@@ -279,32 +291,19 @@ __device__ __forceinline__ bool wait_progress(const int* p, int need, uint32_t p
     return false;
 }
 
-// The same progress words in global memory, ordered at GPU scope, for a ring that spans blocks
-// (grid strip pipeline).  The release orders the hand-off entries stored before it; the acquire
-// orders the entry loads after it.
-__device__ __forceinline__ void publish_progress_gpu(int* p, int v) {
-    asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// Bounded wait for *p >= need; *seen gets the value observed (the caller may then read every
-// entry up to it without another acquire).  False (and the device error word set) when it runs out.
-__device__ __forceinline__ bool wait_progress_gpu(const int* p, int need, int* seen, uint32_t polls) {
+// A counter in global memory, read with acquire at GPU scope (the strip chain's buffers): accesses
+// after the wait come after those that its writer's fence ordered before the count.
+// Bounded wait for *p >= need; false (and the device error word set) when it runs out.
+__device__ __forceinline__ bool wait_progress_gpu(const int* p, int need, uint32_t polls) {
     for (uint32_t it = 0; it < polls; ++it) {
         int v;
         asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-        if (v >= need) {
-            *seen = v;
-            return true;
-        }
+        if (v >= need) return true;
         __nanosleep(64);
     }
     record_error(SK_ERR_DEVICE_TIMEOUT);
     return false;
 }
-
-// Columns a ring spanning blocks publishes at once: a GPU-scope release every step stalls the
-// publishing lane (and so its warp) far longer than the step itself.
-constexpr int kGridPublish = 8;
 
 // Pop the next work item for a warp (lane 0 takes it, all lanes receive it).
 __device__ __forceinline__ int64_t next_item(const Launch& L) {

@@ -7,17 +7,20 @@
 
 #include <cuda_runtime.h>
 
+#include "../../include/sigkernel.h"
+
 namespace sk {
 
-// T: 0 = FP64 cell updates, 1 = FP32; coop: the cooperative-block (strip pipeline) variant,
-// launched with kCoopWarps warps per block; mt: the tiled-M variant (FP32 only).  NULL when no
-// kernel exists for the request.
-// tape: the one-warp-per-pair kernel that records the forward tape (for the approximation scheme
-// a separate instantiation records the derivatives of each cell's outputs with respect to M; the
+// T: 0 = FP64 cell updates, 1 = FP32; chain: the strip-chain variant (a warp per strip, with its own
+// M), else one warp per pair; mt: the tiled-M variant (FP32 only).  NULL when no kernel exists for the request.
+// tape: the kernel that records the forward tape (for the approximation scheme a separate
+// instantiation records the derivatives of each cell's outputs with respect to M; the
 // interpolation kernels record their inputs whenever the launch carries a tape).
 // mx: the FP32 approximation-scheme variant whose cells read M from the buffer the tensor-core M
-// kernel writes (one warp per pair; with tape, recording the tape of output derivatives).
-const void* fwd_poly_kernel_ptr(int T, bool interp, int N, bool coop, bool mt, bool tape = false, bool mx = false);
+// kernel writes (with tape, recording the tape of output derivatives).
+const void* fwd_poly_kernel_ptr(int T, bool interp, int N, bool chain, bool mt, bool tape = false, bool mx = false);
+const void* fwd_approx_chain_tape_ptr_f32(int N);
+const void* fwd_approx_chain_tape_ptr_f64(int N);
 const void* fwd_approx_mx_ptr_f32(int N);
 const void* fwd_approx_tape_mx_ptr_f32(int N);
 const void* fwd_approx_tape_ptr_f32(int N);
@@ -36,47 +39,40 @@ const void* fwd_fd_coop_ptr(int T, int order, int lam);
 const void* fwd_fd_implicit_ptr(int T, int lam, bool coop);  // order 3
 const void* fwd_approx_ptr_f32(int N);
 const void* fwd_interp_ptr_f32(int N);
-const void* fwd_approx_coop_ptr_f32(int N);
-const void* fwd_interp_coop_ptr_f32(int N);
+const void* fwd_approx_chain_ptr_f32(int N);
+const void* fwd_interp_chain_ptr_f32(int N);
 const void* fwd_approx_ptr_f64(int N);
 const void* fwd_interp_ptr_f64(int N);
-const void* fwd_approx_coop_ptr_f64(int N);
-const void* fwd_interp_coop_ptr_f64(int N);
+const void* fwd_approx_chain_ptr_f64(int N);
+const void* fwd_interp_chain_ptr_f64(int N);
 const void* fwd_approx_mt_ptr_f32(int N);
 const void* fwd_interp_mt_ptr_f32(int N);
-const void* fwd_approx_coop_mt_ptr_f32(int N);
-const void* fwd_interp_coop_mt_ptr_f32(int N);
 // interpolation orders are split over several units (chunk k of each family)
 const void* fwd_interp_ptr_f32_0(int N);
 const void* fwd_interp_ptr_f32_1(int N);
 const void* fwd_interp_ptr_f32_2(int N);
 const void* fwd_interp_ptr_f32_3(int N);
 const void* fwd_interp_ptr_f32_4(int N);
-const void* fwd_interp_coop_ptr_f32_0(int N);
-const void* fwd_interp_coop_ptr_f32_1(int N);
-const void* fwd_interp_coop_ptr_f32_2(int N);
-const void* fwd_interp_coop_ptr_f32_3(int N);
-const void* fwd_interp_coop_ptr_f32_4(int N);
+const void* fwd_interp_chain_ptr_f32_0(int N);
+const void* fwd_interp_chain_ptr_f32_1(int N);
+const void* fwd_interp_chain_ptr_f32_2(int N);
+const void* fwd_interp_chain_ptr_f32_3(int N);
+const void* fwd_interp_chain_ptr_f32_4(int N);
 const void* fwd_interp_ptr_f64_0(int N);
 const void* fwd_interp_ptr_f64_1(int N);
 const void* fwd_interp_ptr_f64_2(int N);
 const void* fwd_interp_ptr_f64_3(int N);
 const void* fwd_interp_ptr_f64_4(int N);
-const void* fwd_interp_coop_ptr_f64_0(int N);
-const void* fwd_interp_coop_ptr_f64_1(int N);
-const void* fwd_interp_coop_ptr_f64_2(int N);
-const void* fwd_interp_coop_ptr_f64_3(int N);
-const void* fwd_interp_coop_ptr_f64_4(int N);
+const void* fwd_interp_chain_ptr_f64_0(int N);
+const void* fwd_interp_chain_ptr_f64_1(int N);
+const void* fwd_interp_chain_ptr_f64_2(int N);
+const void* fwd_interp_chain_ptr_f64_3(int N);
+const void* fwd_interp_chain_ptr_f64_4(int N);
 const void* fwd_interp_mt_ptr_f32_0(int N);
 const void* fwd_interp_mt_ptr_f32_1(int N);
 const void* fwd_interp_mt_ptr_f32_2(int N);
 const void* fwd_interp_mt_ptr_f32_3(int N);
 const void* fwd_interp_mt_ptr_f32_4(int N);
-const void* fwd_interp_coop_mt_ptr_f32_0(int N);
-const void* fwd_interp_coop_mt_ptr_f32_1(int N);
-const void* fwd_interp_coop_mt_ptr_f32_2(int N);
-const void* fwd_interp_coop_mt_ptr_f32_3(int N);
-const void* fwd_interp_coop_mt_ptr_f32_4(int N);
 }  // namespace sk
 
 namespace sk {
@@ -97,6 +93,13 @@ const void* bwd_tape_interp_ptr_f32(int N);
 const void* bwd_tape_interp_ptr_f64(int N);
 const void* bwd_tape_interp_ptr_f64_0(int N);
 const void* bwd_tape_interp_ptr_f64_1(int N);
+// The same adjoint with a warp per strip.
+const void* bwd_chain_ptr(int T, int N, bool interp);
+const void* bwd_chain_approx_ptr_f32(int N);
+const void* bwd_chain_approx_ptr_f64(int N);
+const void* bwd_chain_interp_ptr_f32(int N);
+const void* bwd_chain_interp_ptr_f64_0(int N);
+const void* bwd_chain_interp_ptr_f64_1(int N);
 // C: coordinates per contraction pass (8, 16 or 32)
 const void* bwd_contract_ptr_f32(int C);
 const void* bwd_contract_ptr_f64(int C);
@@ -128,6 +131,9 @@ cudaError_t launch_m_tc(int KP, const Launch& L, const void* xt, const void* yt,
 namespace sk {
 // Message returned by sigkernel_last_error() on this host thread (for entry points in other units).
 void set_last_error(const char* msg);
+// Scratch that sigkernel_pairs takes for this call when it is given `capacity` bytes.
+int pairs_need(const sk_paths* X, const sk_paths* Y, int32_t d, int64_t npairs, const sk_options* opt, size_t capacity,
+               size_t* need);
 }  // namespace sk
 
 namespace sk {

@@ -6,21 +6,21 @@ namespace sk {
 
 const void* fwd_approx_mt_ptr_f32(int N) {
     switch (N) {
-        case 2: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 2, 2, false, 1, true>);
-        case 3: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 3, 3, false, 1, true>);
-        case 4: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 4, 4, false, 1, true>);
-        case 5: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 5, 5, false, 1, true>);
-        case 6: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 6, 6, false, 1, true>);
-        case 7: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 7, 7, false, 1, true>);
-        case 8: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 8, 8, false, 1, true>);
-        case 9: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 9, 9, false, 1, true>);
-        case 10: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 10, 10, false, 1, true>);
-        case 11: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 11, 11, false, 1, true>);
-        case 12: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 12, 12, false, 1, true>);
-        case 13: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 13, 13, false, 1, true>);
-        case 14: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 14, 14, false, 1, true>);
-        case 15: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 15, 15, false, 1, true>);
-        case 16: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 16, 16, false, 1, true>);
+        case 2: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 2, 2, false, true>);
+        case 3: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 3, 3, false, true>);
+        case 4: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 4, 4, false, true>);
+        case 5: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 5, 5, false, true>);
+        case 6: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 6, 6, false, true>);
+        case 7: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 7, 7, false, true>);
+        case 8: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 8, 8, false, true>);
+        case 9: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 9, 9, false, true>);
+        case 10: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 10, 10, false, true>);
+        case 11: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 11, 11, false, true>);
+        case 12: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 12, 12, false, true>);
+        case 13: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 13, 13, false, true>);
+        case 14: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 14, 14, false, true>);
+        case 15: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 15, 15, false, true>);
+        case 16: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 16, 16, false, true>);
         default: return nullptr;
     }
 }

@@ -7,7 +7,7 @@ namespace sk {
 
 template <int N>
 const void* mx_kernel() {
-    return reinterpret_cast<const void*>(&fwd_poly_kernel<float, N, N, false, 1, false, false, true>);
+    return reinterpret_cast<const void*>(&fwd_poly_kernel<float, N, N, false, false, false, true>);
 }
 
 const void* fwd_approx_mx_ptr_f32(int N) {

@@ -7,16 +7,16 @@ namespace sk {
 
 const void* fwd_approx_tape_ptr_f32(int N) {
     switch (N) {
-        case 2: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 2, 2, false, 1, false, true>);
-        case 3: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 3, 3, false, 1, false, true>);
-        case 4: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 4, 4, false, 1, false, true>);
-        case 5: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 5, 5, false, 1, false, true>);
-        case 6: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 6, 6, false, 1, false, true>);
-        case 7: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 7, 7, false, 1, false, true>);
-        case 8: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 8, 8, false, 1, false, true>);
-        case 9: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 9, 9, false, 1, false, true>);
-        case 10: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 10, 10, false, 1, false, true>);
-        case 12: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 12, 12, false, 1, false, true>);
+        case 2: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 2, 2, false, false, true>);
+        case 3: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 3, 3, false, false, true>);
+        case 4: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 4, 4, false, false, true>);
+        case 5: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 5, 5, false, false, true>);
+        case 6: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 6, 6, false, false, true>);
+        case 7: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 7, 7, false, false, true>);
+        case 8: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 8, 8, false, false, true>);
+        case 9: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 9, 9, false, false, true>);
+        case 10: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 10, 10, false, false, true>);
+        case 12: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 12, 12, false, false, true>);
         default: return nullptr;
     }
 }

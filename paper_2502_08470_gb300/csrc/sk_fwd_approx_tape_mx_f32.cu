@@ -8,7 +8,7 @@ namespace sk {
 
 template <int N>
 const void* tape_mx_kernel() {
-    return reinterpret_cast<const void*>(&fwd_poly_kernel<float, N, N, false, 1, false, true, true>);
+    return reinterpret_cast<const void*>(&fwd_poly_kernel<float, N, N, false, false, true, true>);
 }
 
 const void* fwd_approx_tape_mx_ptr_f32(int N) {

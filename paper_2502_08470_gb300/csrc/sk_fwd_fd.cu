@@ -23,8 +23,8 @@ const void* fwd_interp_ptr_f32(int N) {
     return nullptr;
 }
 
-const void* fwd_interp_coop_ptr_f32(int N) {
-    if (const void* k = fwd_interp_coop_ptr_f32_0(N)) return k; if (const void* k = fwd_interp_coop_ptr_f32_1(N)) return k; if (const void* k = fwd_interp_coop_ptr_f32_2(N)) return k; if (const void* k = fwd_interp_coop_ptr_f32_3(N)) return k; if (const void* k = fwd_interp_coop_ptr_f32_4(N)) return k;
+const void* fwd_interp_chain_ptr_f32(int N) {
+    if (const void* k = fwd_interp_chain_ptr_f32_0(N)) return k; if (const void* k = fwd_interp_chain_ptr_f32_1(N)) return k; if (const void* k = fwd_interp_chain_ptr_f32_2(N)) return k; if (const void* k = fwd_interp_chain_ptr_f32_3(N)) return k; if (const void* k = fwd_interp_chain_ptr_f32_4(N)) return k;
     return nullptr;
 }
 
@@ -33,8 +33,8 @@ const void* fwd_interp_ptr_f64(int N) {
     return nullptr;
 }
 
-const void* fwd_interp_coop_ptr_f64(int N) {
-    if (const void* k = fwd_interp_coop_ptr_f64_0(N)) return k; if (const void* k = fwd_interp_coop_ptr_f64_1(N)) return k; if (const void* k = fwd_interp_coop_ptr_f64_2(N)) return k; if (const void* k = fwd_interp_coop_ptr_f64_3(N)) return k; if (const void* k = fwd_interp_coop_ptr_f64_4(N)) return k;
+const void* fwd_interp_chain_ptr_f64(int N) {
+    if (const void* k = fwd_interp_chain_ptr_f64_0(N)) return k; if (const void* k = fwd_interp_chain_ptr_f64_1(N)) return k; if (const void* k = fwd_interp_chain_ptr_f64_2(N)) return k; if (const void* k = fwd_interp_chain_ptr_f64_3(N)) return k; if (const void* k = fwd_interp_chain_ptr_f64_4(N)) return k;
     return nullptr;
 }
 
@@ -43,29 +43,23 @@ const void* fwd_interp_mt_ptr_f32(int N) {
     return nullptr;
 }
 
-const void* fwd_interp_coop_mt_ptr_f32(int N) {
-    if (const void* k = fwd_interp_coop_mt_ptr_f32_0(N)) return k; if (const void* k = fwd_interp_coop_mt_ptr_f32_1(N)) return k; if (const void* k = fwd_interp_coop_mt_ptr_f32_2(N)) return k; if (const void* k = fwd_interp_coop_mt_ptr_f32_3(N)) return k; if (const void* k = fwd_interp_coop_mt_ptr_f32_4(N)) return k;
-    return nullptr;
-}
-
-const void* fwd_poly_kernel_ptr(int T, bool interp, int N, bool coop, bool mt, bool tape, bool mx) {
+const void* fwd_poly_kernel_ptr(int T, bool interp, int N, bool chain, bool mt, bool tape, bool mx) {
+    if (chain) {
+        if (tape && !interp) return T == 1 ? fwd_approx_chain_tape_ptr_f32(N) : fwd_approx_chain_tape_ptr_f64(N);
+        if (T == 1) return interp ? fwd_interp_chain_ptr_f32(N) : fwd_approx_chain_ptr_f32(N);
+        return interp ? fwd_interp_chain_ptr_f64(N) : fwd_approx_chain_ptr_f64(N);
+    }
     if (mx) {
-        if (T != 1 || interp || coop) return nullptr;
+        if (T != 1 || interp) return nullptr;
         return tape ? fwd_approx_tape_mx_ptr_f32(N) : fwd_approx_mx_ptr_f32(N);
     }
     if (tape && !interp) {
-        if (coop) return nullptr;
         if (T == 1) return mt ? fwd_approx_tape_ptr_f32_mt(N) : fwd_approx_tape_ptr_f32(N);
         return mt ? nullptr : fwd_approx_tape_ptr_f64(N);
     }
     if (mt) {
         if (T != 1) return nullptr;
-        if (coop) return interp ? fwd_interp_coop_mt_ptr_f32(N) : fwd_approx_coop_mt_ptr_f32(N);
         return interp ? fwd_interp_mt_ptr_f32(N) : fwd_approx_mt_ptr_f32(N);
-    }
-    if (coop) {
-        if (T == 1) return interp ? fwd_interp_coop_ptr_f32(N) : fwd_approx_coop_ptr_f32(N);
-        return interp ? fwd_interp_coop_ptr_f64(N) : fwd_approx_coop_ptr_f64(N);
     }
     if (T == 1) return interp ? fwd_interp_ptr_f32(N) : fwd_approx_ptr_f32(N);
     return interp ? fwd_interp_ptr_f64(N) : fwd_approx_ptr_f64(N);

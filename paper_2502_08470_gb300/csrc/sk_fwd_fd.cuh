@@ -67,8 +67,12 @@ __device__ __forceinline__ T fd_pow2(int e) {
     else return pow2d(e);
 }
 
-// Sweep of one pair by one warp (CW = 1) or by warp w of a cooperative block of CW warps
-// (strips w, w + CW, ...; hand-off ordering as in sweep_poly).
+// Sweep of one pair by one warp (CW = 1) or by warp w of a cooperative block of CW warps (strips w,
+// w + CW, ...).  Lane 31 of strip g writes its top nodes into this warp's hand-off buffer (own_buf);
+// lane 0 of strip g + 1 reads them from the buffer of the warp that ran strip g (prev_buf, the
+// warp's own when CW = 1).  In a block the hand-off is ordered by the progress words prog[]; a buffer
+// entry of strip g is overwritten by strip g + CW only after strip g + 1 has consumed it, because
+// strip g + CW depends on strip g + 1 through the strips in between.
 template <typename T, int ORDER, int R, int CW, bool TAPE = false>
 __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const PairDesc& P, int w, char* own_buf,
                                          const char* prev_buf, int* prog, int64_t buf_cols) {

@@ -6,8 +6,8 @@ namespace sk {
 
 const void* fwd_interp_ptr_f32_2(int N) {
     switch (N) {
-        case 9: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 9, 9 + sk::kJF32, true, 1, false>);
-        case 10: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 10, 10 + sk::kJF32, true, 1, false>);
+        case 9: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 9, 9 + sk::kJF32, true, false>);
+        case 10: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 10, 10 + sk::kJF32, true, false>);
         default: return nullptr;
     }
 }

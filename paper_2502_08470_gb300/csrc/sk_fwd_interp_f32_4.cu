@@ -6,7 +6,7 @@ namespace sk {
 
 const void* fwd_interp_ptr_f32_4(int N) {
     switch (N) {
-        case 12: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 12, 12 + sk::kJF32, true, 1, false>);
+        case 12: return reinterpret_cast<const void*>(&fwd_poly_kernel<float, 12, 12 + sk::kJF32, true, false>);
         default: return nullptr;
     }
 }

@@ -6,11 +6,11 @@ namespace sk {
 
 const void* fwd_interp_ptr_f64_0(int N) {
     switch (N) {
-        case 2: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 2, 2 + sk::kJF64, true, 1, false>);
-        case 3: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 3, 3 + sk::kJF64, true, 1, false>);
-        case 4: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 4, 4 + sk::kJF64, true, 1, false>);
-        case 5: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 5, 5 + sk::kJF64, true, 1, false>);
-        case 6: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 6, 6 + sk::kJF64, true, 1, false>);
+        case 2: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 2, 2 + sk::kJF64, true, false>);
+        case 3: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 3, 3 + sk::kJF64, true, false>);
+        case 4: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 4, 4 + sk::kJF64, true, false>);
+        case 5: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 5, 5 + sk::kJF64, true, false>);
+        case 6: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 6, 6 + sk::kJF64, true, false>);
         default: return nullptr;
     }
 }

@@ -6,8 +6,8 @@ namespace sk {
 
 const void* fwd_interp_ptr_f64_1(int N) {
     switch (N) {
-        case 7: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 7, 7 + sk::kJF64, true, 1, false>);
-        case 8: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 8, 8 + sk::kJF64, true, 1, false>);
+        case 7: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 7, 7 + sk::kJF64, true, false>);
+        case 8: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 8, 8 + sk::kJF64, true, false>);
         default: return nullptr;
     }
 }

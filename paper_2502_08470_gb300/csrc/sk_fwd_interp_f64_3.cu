@@ -6,7 +6,7 @@ namespace sk {
 
 const void* fwd_interp_ptr_f64_3(int N) {
     switch (N) {
-        case 11: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 11, 11 + sk::kJF64, true, 1, false>);
+        case 11: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 11, 11 + sk::kJF64, true, false>);
         default: return nullptr;
     }
 }

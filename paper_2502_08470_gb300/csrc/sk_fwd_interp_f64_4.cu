@@ -6,7 +6,7 @@ namespace sk {
 
 const void* fwd_interp_ptr_f64_4(int N) {
     switch (N) {
-        case 12: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 12, 12 + sk::kJF64, true, 1, false>);
+        case 12: return reinterpret_cast<const void*>(&fwd_poly_kernel<double, 12, 12 + sk::kJF64, true, false>);
         default: return nullptr;
     }
 }

@@ -1,0 +1,14 @@
+// Instantiations of the strip-chain polynomial-interpolation forward wavefront (double cell updates), orders 11..11 (one unit per group of orders so that the units compile in parallel).
+#include "sk_fwd_chain.cuh"
+#include "sk_dispatch.h"
+
+namespace sk {
+
+const void* fwd_interp_chain_ptr_f64_3(int N) {
+    switch (N) {
+        case 11: return reinterpret_cast<const void*>(&fwd_chain_kernel<double, 11, 11 + sk::kJF64, true>);
+        default: return nullptr;
+    }
+}
+
+}  // namespace sk

@@ -1,0 +1,14 @@
+// Instantiations of the strip-chain polynomial-interpolation forward wavefront (double cell updates), orders 12..12 (one unit per group of orders so that the units compile in parallel).
+#include "sk_fwd_chain.cuh"
+#include "sk_dispatch.h"
+
+namespace sk {
+
+const void* fwd_interp_chain_ptr_f64_4(int N) {
+    switch (N) {
+        case 12: return reinterpret_cast<const void*>(&fwd_chain_kernel<double, 12, 12 + sk::kJF64, true>);
+        default: return nullptr;
+    }
+}
+
+}  // namespace sk

@@ -59,6 +59,14 @@ __device__ __forceinline__ void build_exp_series(T M, float tau, T (&e)[NE + 1])
     for (int m = 1; m <= NE; ++m) e[m] = e[m - 1] * (M * Tab<T>::inv(m));
 }
 
+// The series where the caller knows that |M| <= tau (the same values as build_exp_series there).
+template <typename T, int NE>
+__device__ __forceinline__ void build_small_exp_series(T M, T (&e)[NE + 1]) {
+    e[0] = T(1);
+#pragma unroll
+    for (int m = 1; m <= NE; ++m) e[m] = e[m - 1] * (M * Tab<T>::inv(m));
+}
+
 // Broadcast of one FP32 value into both halves of a packed pair.
 __device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
 
@@ -144,6 +152,65 @@ __device__ __forceinline__ void cell_series_dm(const T (&a)[N + 1], const T (&b)
             da[n] = fma(e[n], ta[n + 1], vt);
             db[n] = fma(e[n], tb[n + 1], vr);
         }
+    }
+}
+
+// The approximation cell on edge pairs: the same products and sums as cell_series, bit for bit, with
+// the two edges in the halves of the two-wide FP32 instructions: c_n = (ct_n, cr_n) from (a_k, b_k)
+// (convolution) and (b_k, a_k) (coupling).  Half the multiply-adds to issue for about 30 moves; where
+// issue slots or their latency bind, that is fewer cycles (the strip chain, order 6: 4.88 against
+// 5.15 ms on one pair of 4096 x 4096 cells, 9.65 against 10.8 ms on 48 such pairs).
+template <int N>
+__device__ __forceinline__ void cell_pairs(const float (&a)[N + 1], const float (&b)[N + 1], const float (&e)[N + 1],
+                                           float2 (&c)[N + 1]) {
+    float2 p[N + 1], q[N + 1], e2[N + 1];
+#pragma unroll
+    for (int n = 0; n <= N; ++n) {
+        p[n] = make_float2(a[n], b[n]);
+        q[n] = make_float2(b[n], a[n]);
+        e2[n] = dup2(e[n]);
+    }
+#pragma unroll
+    for (int n = 0; n <= N; ++n) {
+        float2 t = p[0];
+#pragma unroll
+        for (int k = 1; k <= N; ++k) t = __ffma2_rn(q[k], dup2(Tab<float>::hank(n, k)), t);
+        if (n > 0) {
+            float2 v = p[n];
+#pragma unroll
+            for (int k = n - 1; k >= 1; --k) v = __ffma2_rn(p[k], e2[n - k], v);
+            t = __ffma2_rn(e2[n], t, v);
+        }
+        c[n] = t;
+    }
+}
+
+// cell_series_dm on edge pairs: d[n - 1] = (d a'_n / dM, d b'_n / dM).
+template <int N>
+__device__ __forceinline__ void cell_pairs_dm(const float (&a)[N + 1], const float (&b)[N + 1], const float (&e)[N + 1],
+                                              float2 (&c)[N + 1], float2 (&d)[N]) {
+    float2 p[N + 1], q[N + 1], t[N + 1], e2[N + 1];
+#pragma unroll
+    for (int n = 0; n <= N; ++n) {
+        p[n] = make_float2(a[n], b[n]);
+        q[n] = make_float2(b[n], a[n]);
+        e2[n] = dup2(e[n]);
+    }
+#pragma unroll
+    for (int n = 0; n <= N; ++n) {
+        t[n] = p[0];
+#pragma unroll
+        for (int k = 1; k <= N; ++k) t[n] = __ffma2_rn(q[k], dup2(Tab<float>::hank(n, k)), t[n]);
+    }
+    c[0] = t[0];
+    d[0] = t[1];
+#pragma unroll
+    for (int n = 1; n <= N; ++n) {
+        float2 v = p[n];
+#pragma unroll
+        for (int k = n - 1; k >= 1; --k) v = __ffma2_rn(p[k], e2[n - k], v);
+        c[n] = __ffma2_rn(e2[n], t[n], v);
+        if (n < N) d[n] = __ffma2_rn(e2[n], t[n + 1], v);
     }
 }
 
@@ -303,49 +370,20 @@ __device__ __forceinline__ void produce_m_strip(const T* __restrict__ xbase, con
     __syncwarp();  // the strip's M is visible to every lane
 }
 
-// Warps of a block that sweep one long pair together (strip pipeline); see sweep_poly.  Sixteen
-// measured faster than eight both on few long pairs (64 pairs of 1025-point paths: 4.6 against
-// 5.8 ms) and on uneven batches (4096 pairs of 64..4096-point paths: 101 against 121 ms).
-constexpr int kCoopWarps = 16;
-
-template <typename T, int N, int NE, bool MT = false>
-constexpr int fwd_poly_coop_min_blocks() {
-    // Two 16-warp blocks per SM (64 registers) measured faster for the approximation scheme up to
-    // order 6 in FP32, despite a few spilled registers: 4096 pairs of 64..4096-point paths ran in
-    // 83.7 ms against 101.4 ms.  The interpolation scheme's longer series spill more, and it ran
-    // slower that way (64 pairs of 1025-point oscillatory paths: 5.47 against 4.76 ms), so it
-    // keeps one block.
-    if constexpr (std::is_same<T, float>::value && NE == N && N <= 6 && !MT) return 2;
-    constexpr int b = fwd_poly_min_blocks<T, N, NE, MT>() * kFwdWarps / kCoopWarps;
-    return b < 1 ? 1 : b;
-}
-
-// Sweep of one pair by one warp (CW = 1), or by warp w of a ring of `ring` warps that share it:
-// warp w runs strips w, w + ring, w + 2 ring, ... in the same overlapped schedule a single warp
-// uses for all of them (local strip sigma starts at local step sigma * P).  Lane 31 of strip g
-// writes its right edges into this warp's hand-off buffer (own_buf); lane 0 of strip g + 1 reads
-// them from the buffer of the warp that ran strip g (prev_buf, the warp's own buffer when
-// CW = 1).  In a ring the hand-off is ordered by the progress words prog[]; a buffer entry of
-// strip g is overwritten by strip g + ring only after strip g + 1 has consumed it, because strip
-// g + ring depends on strip g + 1 through the chain of strips in between.
-//
-// The ring is the CW warps of one block (ring = CW, progress words in shared memory, CTA-scope
-// ordering), or, with GS, blocks x CW warps spread over co-resident blocks (progress words in
-// global memory, GPU-scope ordering, published every kGridPublish columns).
-template <typename T, int N, int NE, bool INTERP, int CW, bool MT, bool GS = false, bool DMT = false, bool MX = false>
-__device__ __forceinline__ void sweep_poly(const Launch& L, int64_t item, const PairDesc& P, int w, char* own_buf,
-                                           const char* prev_buf, int* prog, int64_t buf_cols, T* xstage,
-                                           int ring = CW) {
+// Sweep of one pair by one warp: strip after strip in the overlapped schedule (strip s starts at
+// step s * P).  Lane 31 writes a strip's right edges into the warp's hand-off buffer; lane 0 reads
+// them for the next strip.
+template <typename T, int N, int NE, bool INTERP, bool MT, bool DMT = false, bool MX = false>
+__device__ __forceinline__ void sweep_poly(const Launch& L, int64_t item, const PairDesc& P, char* own_buf,
+                                           int64_t buf_cols, T* xstage) {
     constexpr bool kRescale = std::is_same<T, float>::value;
-    static_assert(!MX || (CW == 1 && !MT && std::is_same<T, float>::value), "precomputed M: FP32, one warp per pair");
+    static_assert(!MX || (!MT && std::is_same<T, float>::value), "precomputed M: FP32");
     using V = typename Vec<T>::type;
     constexpr int W = Vec<T>::W;
     constexpr int NB = (N + 1 + W - 1) / W * W;  // hand-off entry width, padded to whole vectors
     const int lane = threadIdx.x & 31;
     V* hbuf = reinterpret_cast<V*>(own_buf);                                                // [buf_cols][NB / W]
     int* ebuf = reinterpret_cast<int*>(own_buf + buf_cols * NB * static_cast<int64_t>(sizeof(T)));
-    const V* hprev = reinterpret_cast<const V*>(prev_buf);
-    const int* eprev = reinterpret_cast<const int*>(prev_buf + buf_cols * NB * static_cast<int64_t>(sizeof(T)));
     const int dpad = L.dpad;
     const T* __restrict__ incX = static_cast<const T*>(L.X.inc);
     const T* __restrict__ incY = static_cast<const T*>(L.Y.inc);
@@ -353,24 +391,10 @@ __device__ __forceinline__ void sweep_poly(const Launch& L, int64_t item, const 
     const int lam = L.lam;
     const int rows = static_cast<int>(P.lx << lam);
     const int cols = static_cast<int>(P.ly << lam);
-    // Period of a warp's strips.  Alone, a warp starts its next strip as soon as lane 0 is free
-    // (P = max(cols, 32)).  In a cooperative block that overlap can deadlock: a warp whose lane 0
-    // waits on the ring of other warps also holds back its lanes still publishing the previous
-    // strip, which those warps need.  A warp therefore starts strip k + 1 only after finishing
-    // strip k (P = cols + 31), unless the rows are longer than the ring's lag (cols > 31 CW),
-    // where the overlapped schedule keeps every wait pointed at finished work.  A model of this
-    // schedule (tests/test_pipeline_schedule.py) checks the rule and the deadlock it avoids.
-    // A ring spanning blocks publishes its progress every kGridPublish columns, which lengthens
-    // the lag the overlapped schedule must exceed (the schedule model checks this rule too).
-    constexpr int kLag = GS ? 31 + kGridPublish : 31;
-    const int period = CW == 1 ? (cols > 32 ? cols : 32) : (cols > kLag * ring ? cols : cols + 31);
+    const int period = cols > 32 ? cols : 32;  // a warp starts its next strip as soon as lane 0 is free
     const int nstrips = (rows + 31) >> 5;
-    const int last_lane = (rows - 1) - ((nstrips - 1) << 5);
-    // this warp's strips: w, w + ring, ...; the one holding the last row ends at lane last_lane
-    const int nloc = w < nstrips ? (nstrips - 1 - w) / ring + 1 : 0;
-    if (nloc == 0) return;
-    const bool has_last = (nstrips - 1) % ring == w;
-    const int nsteps = (nloc - 1) * period + (has_last ? last_lane : 31) + cols;
+    const int last_lane = (rows - 1) - ((nstrips - 1) << 5);  // the lane the last strip ends at
+    const int nsteps = (nstrips - 1) * period + last_lane + cols;
     const T sub = pow2t<T>(-2 * lam);  // M of a sub-cell of P_lambda is M_ij / 4^lambda
     const T* xbase = incX + P.xs * dpad;
     const T* ybase = incY + P.ys * dpad;
@@ -379,15 +403,12 @@ __device__ __forceinline__ void sweep_poly(const Launch& L, int64_t item, const 
 #pragma unroll
     for (int n = 0; n <= N; ++n) { a[n] = T(0); bo[n] = T(0); }
     int ea = 0, eo = 0;
-    int jj = -lane, sl = 0;                 // column and local strip of this lane
-    int g = w, row = (w << 5) + lane;       // global strip and grid row
-    bool stuck = false;                     // a hand-off wait ran out (CW > 1 only)
-    int seen = 0;                           // progress of the warp before, as last observed (GS)
+    int jj = -lane, g = 0, row = lane;      // column, strip and grid row of this lane
     const T* xrow = xbase + static_cast<int64_t>(min(row, rows - 1) >> lam) * dpad;
-    // tiled M (MT): this warp's [2][32][mcols] strip buffers; lane 0's column and local strip
+    // tiled M (MT): this warp's [2][32][mcols] strip buffers; lane 0's column and strip
     const int mcols = MT ? L.mtile_cols : 0;
     T* mbuf = MT ? reinterpret_cast<T*>(own_buf + L.mtile_off) : nullptr;
-    int jj0 = 0, sl0 = 0;
+    int jj0 = 0, g0 = 0;
     // precomputed M (MX): this item's groups of four warp steps (lane r's M of steps 4G .. 4G + 3 in
     // the float4 32 G + r).  Group G + 1 is loaded on entering group G, four to seven steps ahead of
     // its use: the groups come from HBM, and a step's cell arithmetic alone does not cover the load
@@ -400,35 +421,26 @@ __device__ __forceinline__ void sweep_poly(const Launch& L, int64_t item, const 
 
     for (int step = 0; step < nsteps; ++step) {
         if constexpr (MT) {
-            if (jj0 == 0 && sl0 < nloc)  // lane 0 enters local strip sl0: build its M first
-                produce_m_strip<T>(xbase, ybase, dpad, lam, rows, cols, w + sl0 * ring, sub, xstage,
-                                   mbuf + (sl0 & 1) * 32 * static_cast<int64_t>(mcols), mcols);
+            if (jj0 == 0 && g0 < nstrips)  // lane 0 enters strip g0: build its M first
+                produce_m_strip<T>(xbase, ybase, dpad, lam, rows, cols, g0, sub, xstage,
+                                   mbuf + (g0 & 1) * 32 * static_cast<int64_t>(mcols), mcols);
             if (++jj0 == period) {
                 jj0 = 0;
-                ++sl0;
+                ++g0;
             }
         }
         T b[N + 1];
 #pragma unroll
         for (int n = 0; n <= N; ++n) b[n] = __shfl_up_sync(kFull, bo[n], 1);
         int eb = kRescale ? __shfl_up_sync(kFull, eo, 1) : 0;
-        const bool active = static_cast<unsigned>(jj) < static_cast<unsigned>(cols) && row < rows && sl < nloc;
+        const bool active = static_cast<unsigned>(jj) < static_cast<unsigned>(cols) && row < rows;
         if (active && lane == 0) {
             if (g == 0) {  // q^{0,j} = e_0 (left boundary k(0, .) = 1)
 #pragma unroll
                 for (int n = 0; n <= N; ++n) b[n] = (n == 0) ? T(1) : T(0);
                 eb = 0;
             } else {
-                if constexpr (CW > 1) {
-                    const int* pp = prog + (w + ring - 1) % ring;
-                    if constexpr (GS) {
-                        const int need = (g - 1) * cols + jj + 1;
-                        if (!stuck && seen < need && !wait_progress_gpu(pp, need, &seen, wait_polls(L))) stuck = true;
-                    } else {
-                        if (!stuck && !wait_progress(pp, (g - 1) * cols + jj + 1, wait_polls(L))) stuck = true;
-                    }
-                }
-                const V* src = hprev + static_cast<int64_t>(jj) * (NB / W);
+                const V* src = hbuf + static_cast<int64_t>(jj) * (NB / W);
 #pragma unroll
                 for (int v = 0; v < NB / W; ++v) {
                     const V t = src[v];
@@ -437,7 +449,7 @@ __device__ __forceinline__ void sweep_poly(const Launch& L, int64_t item, const 
                     for (int q = 0; q < W; ++q)
                         if (v * W + q <= N) b[v * W + q] = tp[q];
                 }
-                if (kRescale) eb = eprev[jj];
+                if (kRescale) eb = ebuf[jj];
             }
         }
         if (active && jj == 0) {  // p^{i,0} = e_0 (bottom boundary k(., 0) = 1)
@@ -461,7 +473,7 @@ __device__ __forceinline__ void sweep_poly(const Launch& L, int64_t item, const 
         // the results of active lanes are ever consumed.
         const int jc = min(max(jj, 0), cols - 1);
         T M;
-        if constexpr (MT) M = active ? mbuf[((sl & 1) * 32 + lane) * static_cast<int64_t>(mcols) + jc] : T(0);
+        if constexpr (MT) M = active ? mbuf[((g & 1) * 32 + lane) * static_cast<int64_t>(mcols) + jc] : T(0);
         else if constexpr (MX) {
             if ((step & 3) == 0) {  // entering group step / 4: its M was read a group ago
                 mcur = mnxt;
@@ -472,7 +484,7 @@ __device__ __forceinline__ void sweep_poly(const Launch& L, int64_t item, const 
             mcur = make_float4(mcur.y, mcur.z, mcur.w, 0.f);
         }
         else M = row_dot<T>(xrow, ybase + static_cast<int64_t>(jc >> lam) * dpad, L.nvec) * sub;
-        if constexpr (CW == 1 && INTERP) {
+        if constexpr (INTERP) {
             if (L.tape != nullptr) {
                 // Interpolation scheme: record the cell's inputs (a, b, exponent, M) for the
                 // adjoint.  A step of the tape is laid out [vector][lane] (16-byte vectors), so
@@ -555,28 +567,19 @@ __device__ __forceinline__ void sweep_poly(const Launch& L, int64_t item, const 
                 dst[v] = t;
             }
             if (kRescale) ebuf[jj] = eo;
-            if constexpr (CW > 1) {
-                if constexpr (GS) {
-                    if ((jj + 1) % kGridPublish == 0 || jj == cols - 1) publish_progress_gpu(prog + w, g * cols + jj + 1);
-                } else {
-                    publish_progress(prog + w, g * cols + jj + 1);
-                }
-            }
         }
         __syncwarp();
         if (++jj == period) {
             jj = 0;
-            ++sl;
-            g += ring;
-            row += 32 * ring;
+            ++g;
+            row += 32;
             xrow = xbase + static_cast<int64_t>(min(row, rows - 1) >> lam) * dpad;
         }
     }
     if constexpr (!INTERP) {
-        // The last cell was the final step of lane `last_lane` in the warp holding the last
-        // strip; for the approximation scheme its outputs are still in (a, bo):
-        // k_hat = 1/2 sum_n (a_n + b_n) / n!.
-        if (has_last && lane == last_lane) {
+        // The last cell was the final step of lane `last_lane`; for the approximation scheme its
+        // outputs are still in (a, bo): k_hat = 1/2 sum_n (a_n + b_n) / n!.
+        if (lane == last_lane) {
             const double v0 = 0.5 * (series_at_one<T, N>(a) + series_at_one<T, N>(bo));
             const double v = kRescale ? ldexp(v0, ea) : v0;
             if (!isfinite(v)) record_error(SK_ERR_NONFINITE);
@@ -607,71 +610,26 @@ __device__ __forceinline__ bool trivial_pair(const Launch& L, int64_t item, cons
     return false;
 }
 
-// Forward wavefront, persistent.  MT: tiled M (produce_m_strip) instead of per-cell inner
-// products.  CW = 1: blocks of kFwdWarps independent warps, one pair per warp.  CW > 1: blocks of
-// CW warps; the block takes pairs of at least L.coop_min_strips strips together (strip pipeline,
-// sweep_poly<..., CW>), and at the first shorter pair (the queue is ordered by cell count, longest
-// first) its warps fall back to one pair each.  DMT (approximation scheme, CW = 1): record the
-// tape of output derivatives with respect to M (L.tape must be set); the interpolation kernels
-// record their tape of cell inputs whenever L.tape is set.  MX (FP32 approximation scheme,
-// CW = 1): the cells read M from the buffer L.mx that the tensor-core M kernel wrote.
-template <typename T, int N, int NE, bool INTERP, int CW, bool MT, bool DMT = false, bool MX = false>
-__global__ void __launch_bounds__((CW > 1 ? CW : kFwdWarps) * 32,
-                                  (CW > 1 ? fwd_poly_coop_min_blocks<T, N, NE, MT>() : fwd_poly_min_blocks<T, N, NE, MT>()))
+// Forward wavefront, persistent: blocks of kFwdWarps independent warps, one pair per warp.  MT: tiled M
+// (produce_m_strip) instead of per-cell inner products.  DMT (approximation scheme): record the tape
+// of output derivatives with respect to M (L.tape must be set); the interpolation kernels record
+// their tape of cell inputs whenever L.tape is set.  MX (FP32 approximation scheme): the cells read M
+// from the buffer L.mx that the tensor-core M kernel wrote.
+template <typename T, int N, int NE, bool INTERP, bool MT, bool DMT = false, bool MX = false>
+__global__ void __launch_bounds__(kFwdWarps * 32, (fwd_poly_min_blocks<T, N, NE, MT>()))
     fwd_poly_kernel(Launch L, int64_t buf_cols) {
     const int wib = threadIdx.x >> 5;
     const int nw = blockDim.x >> 5;
-    char* block_base = static_cast<char*>(L.scratch) + static_cast<int64_t>(blockIdx.x) * nw * L.scratch_stride;
-    char* own = block_base + wib * L.scratch_stride;
+    char* own = static_cast<char*>(L.scratch) + (static_cast<int64_t>(blockIdx.x) * nw + wib) * L.scratch_stride;
     // dynamic shared memory: the x rows of the tiled-M producer ([32][dpad] per warp, with L.mtile)
     extern __shared__ __align__(128) unsigned char fwd_smem[];
     T* xstage = reinterpret_cast<T*>(fwd_smem) + wib * 32 * L.dpad;
-
-    if constexpr (CW > 1) {
-        if (L.grid_bpp > 0) {  // grid strip pipeline: this block is part k of its slot's ring
-            const int bpp = L.grid_bpp;
-            const int64_t slot = blockIdx.x / bpp;
-            const int k = static_cast<int>(blockIdx.x - slot * bpp);
-            if (slot >= L.npairs) return;
-            const int64_t item = L.order ? static_cast<int64_t>(L.order[slot]) : slot;
-            const PairDesc P = decode_pair(L, item);
-            if (trivial_pair(L, item, P)) return;
-            const int ring = bpp * CW;
-            const int wr = k * CW + wib;                 // this warp's place in the ring
-            const int pw = (wr + ring - 1) % ring;       // the warp before it
-            const char* prev = static_cast<char*>(L.scratch) +
-                               ((slot * bpp + pw / CW) * nw + pw % CW) * L.scratch_stride;
-            sweep_poly<T, N, NE, INTERP, CW, MT, true>(L, item, P, wr, own, prev, L.gprog + slot * ring, buf_cols,
-                                                       xstage, ring);
-            return;
-        }
-        __shared__ long long s_item;
-        __shared__ int s_prog[CW];
-        for (;;) {
-            if (threadIdx.x == 0) s_item = pop_item(L);
-            __syncthreads();
-            const int64_t item = s_item;
-            if (threadIdx.x < CW) s_prog[threadIdx.x] = 0;
-            __syncthreads();  // every warp has read s_item and sees the cleared progress words
-            if (item < 0) return;
-            const PairDesc P = decode_pair(L, item);
-            const int nstrips = P.lx > 0 ? static_cast<int>(((P.lx << L.lam) + 31) >> 5) : 0;
-            if (nstrips < L.coop_min_strips) {  // short pairs from here on: one warp each
-                if (wib == 0 && !trivial_pair(L, item, P))
-                    sweep_poly<T, N, NE, INTERP, 1, MT>(L, item, P, 0, own, own, nullptr, buf_cols, xstage);
-                break;
-            }
-            if (!trivial_pair(L, item, P))
-                sweep_poly<T, N, NE, INTERP, CW, MT>(L, item, P, wib, own, block_base + ((wib + CW - 1) % CW) * L.scratch_stride,
-                                                 s_prog, buf_cols, xstage);
-        }
-    }
     for (;;) {
         const int64_t item = next_item(L);
         if (item < 0) break;
         const PairDesc P = decode_pair(L, item);
         if (trivial_pair(L, item, P)) continue;
-        sweep_poly<T, N, NE, INTERP, 1, MT, false, DMT, MX>(L, item, P, 0, own, own, nullptr, buf_cols, xstage);
+        sweep_poly<T, N, NE, INTERP, MT, DMT, MX>(L, item, P, own, buf_cols, xstage);
     }
 }
 

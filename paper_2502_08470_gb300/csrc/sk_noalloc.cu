@@ -25,6 +25,7 @@
 #include <string>
 
 #include "../../include/sigkernel.h"
+#include "sk_dispatch.h"
 
 namespace {
 
@@ -75,7 +76,7 @@ int sigkernel_pairs_noalloc(const sk_paths* X, const sk_paths* Y, int32_t d, int
         addr = g_addr[dev];
     }
     size_t need = 0;
-    int rc = sigkernel_workspace_size(SK_OP_PAIRS, X, Y, d, npairs, opt, &need);
+    int rc = sk::pairs_need(X, Y, d, npairs, opt, kScratchBytes, &need);
     if (rc != SK_OK) return set_error(rc, sigkernel_last_error());
     if (need > kScratchBytes) {
         char buf[256];
