@@ -104,6 +104,10 @@ struct PathSet {
     int64_t count;
     int64_t max_len;         // caller's bound on rows per path
     int64_t rows_total;      // caller's row count
+    // Two sets swept as one (off2 not NULL): paths from `split` on are those of a second set with its
+    // own offsets and bounds, whose increment rows follow the first set's.
+    const int64_t* off2;
+    int64_t split, max_len2, rows2;
 };
 
 struct PairDesc {
@@ -204,14 +208,17 @@ __device__ __forceinline__ int64_t upper_row(int64_t p, int64_t n) {
 
 __device__ __forceinline__ void path_span(const PathSet& S, int64_t a, int inc_mode, int64_t& start,
                                           int64_t& len) {
-    int64_t r0 = S.off[a], r1 = S.off[a + 1];
+    const bool second = S.off2 != nullptr && a >= S.split;
+    const int64_t* off = second ? S.off2 + (a - S.split) : S.off + a;
+    int64_t r0 = off[0], r1 = off[1];
     int64_t rows = r1 - r0;
-    if (r0 < 0 || r1 > S.rows_total || rows < (inc_mode ? 0 : 1) || rows > S.max_len) {
+    if (r0 < 0 || r1 > (second ? S.rows2 : S.rows_total) || rows < (inc_mode ? 0 : 1) ||
+        rows > (second ? S.max_len2 : S.max_len)) {
         start = 0;
         len = -1;
         return;
     }
-    start = r0;
+    start = r0 + (second ? S.rows_total : 0);
     len = inc_mode ? rows : rows - 1;
 }
 
