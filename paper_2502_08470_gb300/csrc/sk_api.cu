@@ -344,6 +344,9 @@ struct Plan {
 
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
+// Dynamic shared memory that every kernel may use without being allowed more: a block's 48 KB less
+// what a kernel declares statically (the strip chain's hand-off buffers).
+constexpr int kPlainSmem = 32 * 1024;
 // Bytes of precomputed M a forward holds at once (the chunk of items whose M the tensor cores
 // wrote before the chunk's sweep); a chunk is a whole number of the sweep's resident warps.
 constexpr size_t kMxBudget = size_t(8) << 30;
@@ -558,7 +561,7 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     };
     auto occupancy = [&](const void* k, int threads, int* per) -> int {
         const int sm = xsmem(threads);
-        if (sm > 48 * 1024) SK_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+        if (sm > kPlainSmem) SK_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
         SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per, k, threads, sm));
         return SK_OK;
     };
@@ -934,7 +937,7 @@ int run_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, 
     }
     int64_t buf_cols = p.buf_cols;
     const int smem = p.smem_x;  // tiled-M x rows
-    if (smem > 48 * 1024) SK_CUDA(cudaFuncSetAttribute(p.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    if (smem > kPlainSmem) SK_CUDA(cudaFuncSetAttribute(p.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const bool timed = (o->flags & SK_FLAG_TIME_KERNEL) != 0;
     if (timed) {
         if (!t_ev0) SK_CUDA(cudaEventCreate(&t_ev0));

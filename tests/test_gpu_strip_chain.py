@@ -34,7 +34,7 @@ def _both(X, Y, pa, pb, **kw):
 
 @pytest.mark.parametrize("scheme,N", [("approx", 2), ("approx", 5), ("approx", 16), ("interp", 4), ("interp", 12)])
 @pytest.mark.parametrize("compute", ["f32", "f64"])
-@pytest.mark.parametrize("lx,ly,d,lam", [(33, 2, 1, 0), (34, 9, 3, 0), (65, 17, 8, 0), (66, 130, 17, 0), (97, 64, 33, 0),
+@pytest.mark.parametrize("lx,ly,d,lam", [(33, 2, 1, 0), (34, 9, 3, 0), (65, 17, 8, 0), (66, 130, 17, 0), (66, 20, 32, 0), (97, 64, 33, 0),
                                          (21, 19, 4, 2)])
 def test_chain_equals_one_warp(scheme, N, compute, lx, ly, d, lam):
     X = _cuda(W.brownian(3, lx, d, seed=1))
