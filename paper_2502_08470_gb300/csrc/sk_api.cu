@@ -94,7 +94,9 @@ struct OwnedWorkspace {
 
 // ------------------------------------------------------------------------------------------
 // Increments dx_i = x_{i+1} - x_i (or the caller's increments) in the compute type, rows
-// zero-padded to `dpad` elements.  One block per path (grid-stride over paths).
+// zero-padded to `dpad` elements.  Grid: paths (strided) x pieces of a path (path_grid).  With one
+// block per path and 64-bit index arithmetic, a path of 16385 points (d = 4) took 316 us and 4096
+// paths of up to 4096 points (d = 16) 420 us.
 // ------------------------------------------------------------------------------------------
 template <typename Tin> __device__ __forceinline__ double load_elem(const Tin* p) { return static_cast<double>(*p); }
 template <> __device__ __forceinline__ double load_elem<__nv_bfloat16>(const __nv_bfloat16* p) {
@@ -108,9 +110,10 @@ __global__ void increments_kernel(const Tin* __restrict__ rows, const int64_t* _
     for (int64_t a = blockIdx.x; a < count; a += gridDim.x) {
         const int64_t r0 = off[a], r1 = off[a + 1], n = r1 - r0;
         if (r0 < 0 || r1 > rows_total || n < (inc_mode ? 0 : 1) || n > max_len) continue;
-        const int64_t len = inc_mode ? n : n - 1;
-        for (int64_t idx = threadIdx.x; idx < len * dpad; idx += blockDim.x) {
-            const int64_t i = idx / dpad;
+        // (rows per path <= kMaxRefined and dpad <= kDMax, so the element index fits 32 bits)
+        const unsigned total = static_cast<unsigned>(inc_mode ? n : n - 1) * dpad;
+        for (unsigned idx = blockIdx.y * blockDim.x + threadIdx.x; idx < total; idx += gridDim.y * blockDim.x) {
+            const unsigned i = idx / dpad;
             const int c = static_cast<int>(idx - i * dpad);
             double v = 0.0;
             if (c < d) {
@@ -303,6 +306,13 @@ __global__ void chain_clear_kernel(uint4* hand, const unsigned long long* used, 
 // ------------------------------------------------------------------------------------------
 // Argument checks and workspace planning.
 // ------------------------------------------------------------------------------------------
+// Whether ordering the items by cell count can matter: not when every path is as long as the longest
+// (as many rows as that takes).  The order is a schedule only; results do not depend on it.
+bool uneven_lengths(const sk_paths* S) { return S->rows_total < S->count * S->max_len; }
+bool sort_items(const sk_paths* X, const sk_paths* Y, const sk_options* o, int64_t items) {
+    return !(o->flags & SK_FLAG_NO_SORT) && items > 1 && (uneven_lengths(X) || uneven_lengths(Y));
+}
+
 // Strip chain of a launch (sk_chain.cuh).
 struct ChainPlan {
     bool on;
@@ -704,11 +714,19 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     return SK_OK;
 }
 
+// Blocks of 128 threads over every element of a path set's rows: paths, and as many pieces of a path as
+// give the GPU about 16 such blocks per SM, at four elements a thread or more.
+dim3 path_grid(const sk_paths* S, int width) {
+    const int64_t x = std::min<int64_t>(S->count, 65535);
+    const int64_t y = std::min<int64_t>((S->max_len * width + 511) / 512, std::max<int64_t>(2432 / x, 1) * 2);
+    return dim3(static_cast<unsigned>(x), static_cast<unsigned>(std::max<int64_t>(y, 1)));
+}
+
 template <typename T>
 int launch_increments(const sk_paths* S, int32_t d, int32_t dtype, int inc_mode, int dpad, void* out,
                       cudaStream_t st) {
     if (S->count == 0) return SK_OK;
-    int blocks = static_cast<int>(S->count < 65535 ? S->count : 65535);
+    const dim3 blocks = path_grid(S, dpad);
     T* o = static_cast<T*>(out);
     switch (dtype) {
         case SK_F64:
@@ -967,7 +985,7 @@ int run_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, 
         SK_CUDA(cudaMemsetAsync(base + p.off_queue, 0, 256 + align256(2 * 65 * sizeof(unsigned int)), st));
         if (p.chain.on) {
             if ((rc = launch_chain_tickets(p.chain, C, !(o->flags & SK_FLAG_NO_SORT), base, p.off_hist, p.off_order, st)) != SK_OK) return rc;
-        } else if (!(o->flags & SK_FLAG_NO_SORT) && n > 1) {
+        } else if (sort_items(X, Y, o, n)) {
             unsigned int* hist = reinterpret_cast<unsigned int*>(base + p.off_hist);
             int32_t* order = reinterpret_cast<int32_t*>(base + p.off_order);
             int sb = static_cast<int>((n + 255) / 256);
@@ -1008,8 +1026,9 @@ __global__ void inc_to_row_grad_kernel(const double* __restrict__ ginc, const in
     for (int64_t a = blockIdx.x; a < count; a += gridDim.x) {
         const int64_t r0 = off[a], r1 = off[a + 1], n = r1 - r0;
         if (r0 < 0 || r1 > rows_total || n < (inc_mode ? 0 : 1) || n > max_len) continue;
-        for (int64_t idx = threadIdx.x; idx < n * d; idx += blockDim.x) {
-            const int64_t p = idx / d;
+        const unsigned total = static_cast<unsigned>(n) * d;
+        for (unsigned idx = blockIdx.y * blockDim.x + threadIdx.x; idx < total; idx += gridDim.y * blockDim.x) {
+            const unsigned p = idx / d;
             const int c = static_cast<int>(idx - p * d);
             double v;
             if (inc_mode) {
@@ -1131,7 +1150,7 @@ int launch_backward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dty
     B.off_rexp = b.off_rexp;
     B.off_ybar = b.off_ybar;
     SK_CUDA(cudaMemsetAsync(base + p.off_queue, 0, 256 + align256(2 * 65 * sizeof(unsigned int)), st));
-    if (!(o->flags & SK_FLAG_NO_SORT) && npairs > 1) {
+    if (sort_items(X, Y, o, npairs)) {
         unsigned int* hist = reinterpret_cast<unsigned int*>(base + p.off_hist);
         int32_t* order = reinterpret_cast<int32_t*>(base + p.off_order);
         int sb = static_cast<int>(std::min<int64_t>((npairs + 255) / 256, 4096));
@@ -1159,8 +1178,7 @@ int launch_backward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dty
 int convert_grad(const sk_paths* S, int32_t d, int dpad, int inc_mode, const double* ginc, double* grad,
                  cudaStream_t st) {
     if (!grad || S->count == 0) return SK_OK;
-    int blocks = static_cast<int>(S->count < 65535 ? S->count : 65535);
-    inc_to_row_grad_kernel<<<blocks, 128, 0, st>>>(ginc, S->offsets, S->count, S->rows_total, S->max_len, d, dpad,
+    inc_to_row_grad_kernel<<<path_grid(S, d), 128, 0, st>>>(ginc, S->offsets, S->count, S->rows_total, S->max_len, d, dpad,
                                                    inc_mode, grad);
     SK_CUDA(cudaGetLastError());
     return SK_OK;
@@ -1404,7 +1422,7 @@ int launch_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int32_
     SK_CUDA(cudaMemsetAsync(base + p.off_queue, 0, 256 + align256(2 * 65 * sizeof(unsigned int)), st));
     if (b.chain.on) {
         if ((rc = launch_chain_tickets(b.chain, L, !(o->flags & SK_FLAG_NO_SORT), base, p.off_hist, p.off_order, st)) != SK_OK) return rc;
-    } else if (!(o->flags & SK_FLAG_NO_SORT) && npairs > 1) {
+    } else if (sort_items(X, Y, o, npairs)) {
         unsigned int* hist = reinterpret_cast<unsigned int*>(base + p.off_hist);
         int32_t* order = reinterpret_cast<int32_t*>(base + p.off_order);
         int sb = static_cast<int>(std::min<int64_t>((npairs + 255) / 256, 4096));
