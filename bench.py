@@ -126,7 +126,7 @@ def load_hbm_peak():
 # 129-point paths (profiles/*_gram48x129.md): both kernels' traffic is per warp step, so it
 # scales with the steps of the bench's Gram.  None when no capture of the current kernel exists.
 NCU_TRAFFIC_RATIO = {"bwd_tape_kernel<float,6,false>": (2.270 + 0.185) / 2.402,
-                     "fwd_poly_kernel<float,6,6,false,1,false,true,true>": (2.207 + 0.161) / 2.242}
+                     "fwd_poly_kernel<float,6,6,false,false,true,true>": (2.207 + 0.161) / 2.242}
 
 
 def parse():
@@ -502,10 +502,10 @@ def main():
     kb = statistics.mean(kb_ms)
     bcall = statistics.mean(run.backward_call_ms) if run.backward_call_ms else None
     tape_gb = tape_buf[0].numel() / 1e9
-    fwd_rl = kernel_roofline("m_tc_kernel<16> + fwd_poly_kernel<float,6,6,false,1,false,true,true> (forward "
+    fwd_rl = kernel_roofline("m_tc_kernel<16> + fwd_poly_kernel<float,6,6,false,false,true,true> (forward "
                              "recording the tape, M from the tensor cores; algorithmic bytes: the tape)", kf,
                              tape_forward_flops_per_cell(DEGREE, D) * cells, tape_forward_bytes(nx * nx, npts), p32,
-                             "fwd_poly_kernel<float,6,6,false,1,false,true,true>")
+                             "fwd_poly_kernel<float,6,6,false,false,true,true>")
     bwd_rl = kernel_roofline("bwd_tape_kernel<float,6,false> (adjoint wavefront from the tape)", kb,
                              tape_adjoint_flops_per_cell(DEGREE) * cells, tape_adjoint_bytes(nx * nx, npts), p32,
                              "bwd_tape_kernel<float,6,false>")
@@ -602,7 +602,7 @@ def main():
         kfo = statistics.mean(kff)
         line["forward_only"] = {"value": cells / (statistics.mean(sf) / 1e3), "unit": "cell-updates/s",
                                 "ms_per_step": statistics.mean(sf),
-                                "kernel": kernel_roofline("m_tc_kernel<16> + fwd_poly_kernel<float,6,6,false,1,false,"
+                                "kernel": kernel_roofline("m_tc_kernel<16> + fwd_poly_kernel<float,6,6,false,false,"
                                                           "false,true> (no tape, M from the tensor cores)", kfo,
                                                           flops_per_cell(DEGREE, D) * cells, 0, p32)}
 
@@ -615,11 +615,11 @@ def main():
         line["fp64_plain_wavefront"] = {
             "forward": {"value": cells / (statistics.mean(s64) / 1e3), "unit": "cell-updates/s",
                         "ms_per_step": statistics.mean(s64),
-                        "kernel": kernel_roofline("fwd_poly_kernel<double,6,6,false,1,false>", k64avg,
+                        "kernel": kernel_roofline("fwd_poly_kernel<double,6,6,false,false>", k64avg,
                                                   flops_per_cell(DEGREE, D) * cells, 0, p64)},
             "fwd_bwd": {"value": cells / (statistics.mean(fb64) / 1e3), "unit": "cell-updates/s",
                         "ms_per_step": statistics.mean(fb64), "tape_gb": round(tape_buf[0].numel() / 1e9, 2),
-                        "forward_kernel": kernel_roofline("fwd_poly_kernel<double,6,6,false,1,false,true>",
+                        "forward_kernel": kernel_roofline("fwd_poly_kernel<double,6,6,false,false,true>",
                                                           statistics.mean(kf64),
                                                           tape_forward_flops_per_cell(DEGREE, D) * cells,
                                                           tape_forward_bytes(nx * nx, npts, esize=8), p64),
@@ -738,7 +738,7 @@ def main():
         line["gram_fd"] = fd
         del Gf
 
-    if "osc" in args.parts:  # 64 pairs of 1025-point oscillatory paths, d=4 (few long pairs: strip pipeline)
+    if "osc" in args.parts:  # 64 pairs of 1025-point oscillatory paths, d=4 (few long pairs: strip chain)
         Xo_np = W.oscillatory(64, 1025, 4, seed=5 + 1000 * rank)
         Yo_np = W.oscillatory(64, 1025, 4, seed=6 + 1000 * rank)
         Xo = torch.tensor(Xo_np, device=dev)
@@ -787,7 +787,7 @@ def main():
         line["long_pair"] = {"workload": "1 pair of 16385-point Brownian paths, d=4, approx N=6, FP32: the pair's "
                                          "512 strips swept by a ring of 32 co-resident 16-warp blocks",
                              "cells": cells_l, "ms": t_grid, "cell_updates_per_s": cells_l / (t_grid / 1e3),
-                             "oracle_check": "a pair of 4097-point prefixes in the same grid strip pipeline"}
+                             "oracle_check": "a pair of 4097-point prefixes in the same strip chain"}
         del Xl, Yl
 
     if "uneven" in args.parts:  # 4096 pairs, lengths log-uniform in [64, 4096], d=16, BF16: autotuned + graph

@@ -104,18 +104,20 @@ enum {
     SK_FLAG_NO_SORT = 8,      /* process pairs in the given order (no cell-count ordering) */
     SK_FLAG_TIME_KERNEL = 16, /* record CUDA events around the wavefront kernel(s) of this call on
                                  `stream`; read the duration with sigkernel_last_kernel_ms() */
-    SK_FLAG_STRIP_PIPELINE = 32,    /* forward: sweep every pair of 2 or more strips (32 grid rows
-                                       each) with a block of warps, one strip per warp in a
-                                       pipeline, instead of one warp per pair */
-    SK_FLAG_NO_STRIP_PIPELINE = 64, /* forward: always one warp per pair.  With neither flag the
-                                       library pipelines every pair of 2 or more strips when some
-                                       pair has 32 or more strips and the batch is too small to
-                                       fill the GPU with one warp per pair.  Neither applies to the
-                                       tape forward or to the adjoints (one warp per pair).  With
-                                       so few pairs that each pair's 16-warp ring can span 8 or
-                                       more blocks, the pipelined polynomial forward spreads each
-                                       ring over co-resident blocks (a cooperative launch; the
-                                       results are the same bit for bit) */
+    SK_FLAG_STRIP_PIPELINE = 32,    /* sweep every pair of 2 or more strips (32 grid rows each) by
+                                       several warps, one strip per warp at a time, instead of one
+                                       warp per pair: the polynomial schemes' strip chain (every
+                                       strip a work item of its own; forward, tape forward and tape
+                                       adjoint), the FD forward's pipelined block of 16 warps */
+    SK_FLAG_NO_STRIP_PIPELINE = 64, /* always one warp per pair.  With neither flag the library
+                                       decides: the strip chain when the batch has too few pairs, or
+                                       too uneven ones, to keep the GPU busy with one warp per pair;
+                                       the FD pipeline when some pair has 32 or more strips and the
+                                       batch is too small to fill the GPU.  The values are the same
+                                       bit for bit where M is formed the same way (see
+                                       SK_FLAG_NO_TC).  A chain needs workspace for its hand-off (at
+                                       most 8 GiB); in a smaller workspace the call uses fewer
+                                       buffers, or one warp per pair */
     SK_FLAG_NO_TILED_M = 128,       /* forward, polynomial schemes in FP32, where the tensor cores
                                        do not compute M (see SK_FLAG_NO_TC): form each cell's M
                                        from its two increment rows.  By default, with d > 8, each
@@ -127,7 +129,7 @@ enum {
                                        adjoint from chunked forward tapes */
     SK_FLAG_NO_TC = 512             /* FP32: keep the tensor cores out.  By default (1) the
                                        approximation scheme's forward with one warp per pair
-                                       (plain or recording a tape; not the strip pipeline) with
+                                       (plain or recording a tape; not the strip chain) with
                                        4 < d <= 32 takes each cell's M_ij = <dx_i, dy_j> /
                                        4^lambda from a tcgen05 GEMM of the increments, run per
                                        chunk of pairs before the chunk's sweep (flag set: tiled
@@ -277,8 +279,8 @@ int sigkernel_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int
  * sigkernel_autotune -- choose the launch shape of a forward call (sigkernel_pairs when pair_a is
  * non-NULL, else sigkernel_gram; same arguments) by timing the candidates on these inputs:
  * one warp per pair in blocks of 1, 2 or 4 warps (each with and without the tiled M where it
- * applies), and the strip pipeline (blocks of 16 warps sharing each pair of two or more strips)
- * when some pair spans two strips.  Each candidate runs
+ * applies), and the strip pipeline (SK_FLAG_STRIP_PIPELINE: several warps share each pair of two or
+ * more strips) when some pair spans two strips.  Each candidate runs
  * once to warm up, then `trials` (1..1000) timed times on `stream`; `out` is overwritten with the
  * results.  The call allocates its own workspace (stream-ordered) and returns after the runs have
  * finished on the device.
@@ -387,8 +389,9 @@ int sigkernel_device_status(void* stream);
 float sigkernel_last_kernel_ms(void);
 
 /*
- * sigkernel_set_wait_limit -- how many times a strip-pipeline hand-off wait polls its progress word
- * (each poll followed by a ~64 ns sleep) before it gives up: the warp then records
+ * sigkernel_set_wait_limit -- how many times a wait for another warp's hand-off polls (each poll
+ * followed by a 32 to 64 ns sleep; a strip of a chain polls as often again for every strip before
+ * it) before it gives up: the warp then records
  * SK_ERR_DEVICE_TIMEOUT in the device error word, finishes its sweep without waiting (that pair's
  * result is then wrong) and the kernel returns normally.  0 restores the default, 2^20 polls.
  * Process-wide; calls launched after it use the new limit.  The paper has no counterpart: this

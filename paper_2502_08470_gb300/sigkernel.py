@@ -30,8 +30,8 @@ FLAG_STRIP_PIPELINE, FLAG_NO_STRIP_PIPELINE, FLAG_NO_TILED_M, FLAG_CHECKPOINT, F
 
 
 def _pipe_flags(strip_pipeline) -> int:
-    """None: the library decides; True: every pair of 2+ strips is swept by a block of warps;
-    False: one warp per pair."""
+    """None: the library decides; True: every pair of 2+ strips is swept by several warps, a strip
+    each; False: one warp per pair."""
     if strip_pipeline is None:
         return 0
     return FLAG_STRIP_PIPELINE if strip_pipeline else FLAG_NO_STRIP_PIPELINE
