@@ -16,6 +16,7 @@
 #include "sk_bwd_poly.cuh"
 #include "sk_chain.cuh"
 #include "sk_fwd_chain.cuh"
+#include "sk_fwd_split.cuh"
 #include "sk_common.cuh"
 #include "sk_dispatch.h"
 
@@ -332,6 +333,7 @@ struct Plan {
     int threads;         // threads per block
     int blocks;          // persistent grid
     bool coop;           // cooperative-block kernel (strip pipeline for long pairs)
+    bool split;          // four warps per pair (FP64, pairs of one strip)
     int coop_min_strips; // strips from which a pair is swept by a whole block
     ChainPlan chain;     // polynomial schemes: a warp per strip instead of one per pair
     bool mtile;          // tiled M (wide increments, polynomial schemes)
@@ -560,6 +562,7 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     }
     p.threads = (wpb_req ? wpb_req : kFwdWarps) * 32;
     p.coop = false;
+    p.split = false;
     p.coop_min_strips = 0;
     p.chain = ChainPlan{};
     const int esize = p.T ? 4 : 8;
@@ -607,9 +610,24 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     }
     bool want_chain = false;
     const int64_t strips = (max_rows + 31) / 32;
-    if (poly && chain_limit > 0 && pipe_req >= 0 && wpb_req == 0 && strips >= 2 && npairs > 0) {
+    if (poly && chain_limit > 0 && pipe_req >= 0 && strips >= 2 && npairs > 0) {
         want_chain = pipe_req > 0 || chain_pays(X, Y, points, lam, npairs, strips, max_cols,
                                                 static_cast<int64_t>(sms) * per_sm * kFwdWarps, p.T);
+    }
+    // FP64 pairs of one strip, no more of them than SMs: four warps share a pair's cells, since one warp
+    // has only a quarter of its SM's FP64 units (sk_fwd_split.cuh).  With two pairs per SM the units
+    // would be shared all the same, and the exchange between the warps would only cost.
+    const bool shape_asked = o->warps_per_block != 0 || (o->flags & (SK_FLAG_STRIP_PIPELINE | SK_FLAG_NO_STRIP_PIPELINE));
+    if (poly && !p.T && allow_coop && !shape_asked && strips == 1 && npairs > 0 && npairs <= sms) {
+        const void* sk = fwd_split_ptr_f64(o->scheme == SK_POLY_INTERP, o->degree);
+        int sper = 0;
+        if (sk && (rc = occupancy(sk, kSplitWarps * 32, &sper)) != SK_OK) return rc;
+        if (sk && sper >= 1) {
+            p.kern = sk;
+            p.split = true;
+            p.threads = kSplitWarps * 32;
+            per_sm = sper;
+        }
     }
     // Tensor-core M: in place of the per-cell or tiled M, the FP32 approximation scheme's
     // one-warp-per-pair sweep reads each cell's M from a buffer that a tcgen05 GEMM fills per chunk
@@ -673,7 +691,7 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
         }
     }
     const int wpb = p.threads / 32;
-    int64_t want = p.coop ? npairs : ((p.chain.on ? p.chain.cap : npairs) + wpb - 1) / wpb;
+    int64_t want = p.coop || p.split ? npairs : ((p.chain.on ? p.chain.cap : npairs) + wpb - 1) / wpb;
     int64_t cap = static_cast<int64_t>(sms) * per_sm;
     p.blocks = static_cast<int>(want < cap ? (want > 0 ? want : 1) : cap);
     p.buf_cols = (Y->max_len << lam) + 1;
@@ -1001,7 +1019,7 @@ int run_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, 
             SK_CUDA(launch_m_tc(p.kp, C, base + p.off_xt, base + p.off_yt, p.xt_nblk, p.yt_nblk,
                                 reinterpret_cast<float*>(base + p.off_mx), p.mx_stride, sms, st));
         void* args[] = {&C, &buf_cols};
-        const int64_t want = p.coop ? n : ((p.chain.on ? p.chain.cap : n) + wpb - 1) / wpb;
+        const int64_t want = p.coop || p.split ? n : ((p.chain.on ? p.chain.cap : n) + wpb - 1) / wpb;
         const int blocks = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(want, p.blocks)));
         SK_CUDA(cudaLaunchKernel(p.kern, dim3(blocks), dim3(p.threads), args, smem, st));
     }

@@ -21,6 +21,8 @@ namespace sk {
 const void* fwd_poly_kernel_ptr(int T, bool interp, int N, bool chain, bool mt, bool tape = false, bool mx = false);
 const void* fwd_approx_chain_tape_ptr_f32(int N);
 const void* fwd_approx_chain_tape_ptr_f64(int N);
+// FP64, orders 2..8: four warps per pair of one strip, each with some of every cell's outputs.
+const void* fwd_split_ptr_f64(bool interp, int N);
 const void* fwd_approx_mx_ptr_f32(int N);
 const void* fwd_approx_tape_mx_ptr_f32(int N);
 const void* fwd_approx_tape_ptr_f32(int N);
