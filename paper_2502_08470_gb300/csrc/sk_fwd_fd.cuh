@@ -30,8 +30,8 @@
 // everything else a step does: exponents, shuffles, the inner product, index arithmetic and the
 // hand-off (209 issue slots per warp step of 4 sub-cells a lane at lambda = 2).  A step of R x C
 // sub-cells pays for these once and forms the one m they share once.  Measured: FD2, lambda = 2,
-// 128 x 128 Gram of 129-point paths, d = 8, FP32, 6.24 -> 2.87 ms with 4 columns a step, 170 warp
-// instructions a step at 0.76 issued a cycle: bound by issue.  FD2, lambda = 1, 48 x 48 pairs, forward
+// 128 x 128 Gram of 129-point paths, d = 8, FP32, 6.24 -> 2.87 ms with 4 columns a step, 302 warp
+// instructions a step (112 of them the 16 sub-cells) at 0.76 issued a cycle: bound by issue.  FD2, lambda = 1, 48 x 48 pairs, forward
 // with tape and adjoint: 1.63 -> 1.02 ms with 2 columns a step, whose tape is half as long.
 #pragma once
 
