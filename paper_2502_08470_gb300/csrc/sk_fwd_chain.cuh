@@ -67,6 +67,7 @@ __device__ __forceinline__ void sweep_strip(const Launch& L, int64_t item, const
     constexpr int W = Vec<T>::W;
     const int lane = threadIdx.x & 31;
     const int dpad = L.dpad;
+    const int row_bytes = dpad * static_cast<int>(sizeof(T));
     const int lam = L.lam;
     const int rows = static_cast<int>(P.lx << lam);
     const int cols = static_cast<int>(P.ly << lam);
@@ -163,7 +164,7 @@ __device__ __forceinline__ void sweep_strip(const Launch& L, int64_t item, const
             Mnext = mring[((t + 1) & (kChainMSteps - 1)) * 32 + ((lane + t + 1) & 31)];
         } else {
             const int jc = min(max(jj, 0), cols - 1);
-            M = row_dot<T>(xrow, ybase + static_cast<int64_t>(jc >> lam) * dpad, L.nvec) * sub;
+            M = row_dot<T>(xrow, row_at(ybase, jc >> lam, row_bytes), L.nvec) * sub;
         }
         if constexpr (INTERP) {
             if (L.tape != nullptr && active) {  // the cell's inputs (layout as in sweep_poly)

@@ -31,8 +31,10 @@
 // hand-off (209 issue slots per warp step of 4 sub-cells a lane at lambda = 2).  A step of R x C
 // sub-cells pays for these once and forms the one m they share once.  Measured: FD2, lambda = 2,
 // 128 x 128 Gram of 129-point paths, d = 8, FP32, 6.24 -> 2.87 ms with 4 columns a step, 302 warp
-// instructions a step (112 of them the 16 sub-cells) at 0.76 issued a cycle: bound by issue.  FD2, lambda = 1, 48 x 48 pairs, forward
-// with tape and adjoint: 1.63 -> 1.02 ms with 2 columns a step, whose tape is half as long.
+// instructions a step (112 of them the 16 sub-cells) at 0.76 issued a cycle: bound by issue.  Inner
+// products without a loop (2.55 ms) and the row's index, test and increments kept over a strip instead
+// of formed each step (2.35 ms) took more of them out.  FD2, lambda = 1, 48 x 48 pairs, forward with
+// tape and adjoint: 1.63 -> 1.02 ms with 2 columns a step, whose tape is half as long, now 0.91 ms.
 #pragma once
 
 #include <type_traits>
@@ -83,6 +85,7 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
     const T* hprev = reinterpret_cast<const T*>(prev_buf);
     const int* eprev = reinterpret_cast<const int*>(hprev + buf_cols);
     const int dpad = L.dpad;
+    const int row_bytes = dpad * static_cast<int>(sizeof(T));
     const T* __restrict__ incX = static_cast<const T*>(L.X.inc);
     const T* __restrict__ incY = static_cast<const T*>(L.Y.inc);
 
@@ -117,6 +120,9 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
 #pragma unroll
     for (int c = 0; c < C; ++c) top[c] = T(0);
     int jj = -lane, sl = 0, gs = w;     // tile, local strip, global strip
+    int g = (w << 5) + lane;            // row group
+    bool row_ok = g < groups;           // the lane has a row in its current strip
+    const T* xrow = xbase + static_cast<int64_t>((min(g, groups - 1) * R) >> lam) * dpad;
     bool stuck = false;
 
     for (int step = 0; step < nsteps; ++step) {
@@ -124,8 +130,7 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
 #pragma unroll
         for (int c = 0; c < C; ++c) kb[c] = __shfl_up_sync(kFull, top[c], 1);
         int eb = kRescale ? __shfl_up_sync(kFull, eo, 1) : 0;
-        const int g = (gs << 5) + lane;
-        const bool active = jj >= 0 && jj < nJ && g < groups && sl < nloc;
+        const bool active = static_cast<unsigned>(jj) < static_cast<unsigned>(nJ) && row_ok;
         if (active) {
             if (lane == 0) {
                 if (gs == 0) {                               // row 0: k(s_0, .) = 1
@@ -161,8 +166,7 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
                     ea = eb;
                 }
             }
-            const T m = row_dot<T>(xbase + static_cast<int64_t>((g * R) >> lam) * dpad,
-                                   ybase + static_cast<int64_t>((jj * C) >> lam) * dpad, L.nvec) * sub;
+            const T m = row_dot<T>(xrow, row_at(ybase, (jj * C) >> lam, row_bytes), L.nvec) * sub;
             if constexpr (TAPE) {  // the tile's inputs for the adjoint (fd_tape_row)
                 using V = typename Vec<T>::type;
                 constexpr int W = Vec<T>::W;
@@ -255,6 +259,9 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
             jj = 0;
             ++sl;
             gs += CW;
+            g += 32 * CW;
+            row_ok = g < groups && sl < nloc;
+            xrow = xbase + static_cast<int64_t>((min(g, groups - 1) * R) >> lam) * dpad;
         }
     }
 }

@@ -385,6 +385,7 @@ __device__ __forceinline__ void sweep_poly(const Launch& L, int64_t item, const 
     V* hbuf = reinterpret_cast<V*>(own_buf);                                                // [buf_cols][NB / W]
     int* ebuf = reinterpret_cast<int*>(own_buf + buf_cols * NB * static_cast<int64_t>(sizeof(T)));
     const int dpad = L.dpad;
+    const int row_bytes = dpad * static_cast<int>(sizeof(T));
     const T* __restrict__ incX = static_cast<const T*>(L.X.inc);
     const T* __restrict__ incY = static_cast<const T*>(L.Y.inc);
 
@@ -483,7 +484,7 @@ __device__ __forceinline__ void sweep_poly(const Launch& L, int64_t item, const 
             M = active ? mcur.x : T(0);
             mcur = make_float4(mcur.y, mcur.z, mcur.w, 0.f);
         }
-        else M = row_dot<T>(xrow, ybase + static_cast<int64_t>(jc >> lam) * dpad, L.nvec) * sub;
+        else M = row_dot<T>(xrow, row_at(ybase, jc >> lam, row_bytes), L.nvec) * sub;
         if constexpr (INTERP) {
             if (L.tape != nullptr) {
                 // Interpolation scheme: record the cell's inputs (a, b, exponent, M) for the
