@@ -1110,7 +1110,8 @@ __global__ void __launch_bounds__(kFwdWarps * 32, (bwd_tape_min_blocks<T, N, INT
 //   * dk/dx: lane r walks its row (q = 0..31) against the dy rows;
 //   * dk/dy: lane q walks its column (r = 0..31) against the broadcast dx rows;
 // both conflict-free in FP32, every operand in shared memory, each cell's dk/dM read once for all
-// C coordinates, and the products as two-wide FP32 instructions.  Row sums stay in registers
+// C coordinates, and the products as two-wide FP32 instructions.  (FP32 with C = 8 cuts the tile into
+// blocks of cells instead, contract_block.)  Row sums stay in registers
 // across a strip's tiles and go to the FP64 gradients once per strip (strips own disjoint rows).
 // Column sums are added to a shared per-column accumulator once per tile; the columns are taken a
 // window at a time (as many as the accumulator holds), and the accumulator goes to the FP64
@@ -1120,12 +1121,17 @@ constexpr int kContractWarps = 4;
 constexpr int kContractSlack = 64;  // buffer rows past an item's last step that a tile may read
 constexpr int kContractAccBytes = 32 << 10;  // per-block column accumulator
 
+// FP32 with up to 8 coordinates: a lane takes a block of the tile's cells (contract_block).
+template <typename T, int C>
+__host__ __device__ constexpr bool contract_blocked() { return C == 8 && std::is_same<T, float>::value; }
+
 // Shared memory of one contraction warp, padded to 128 bytes so that every warp's ring (a bulk
 // copy destination) starts 128-byte aligned.
 template <typename T, int C>
 __host__ __device__ constexpr int contract_warp_bytes() {
     return (3 * 32 * 32 * static_cast<int>(sizeof(T))    // ring of three halves
             + 2 * 32 * C * static_cast<int>(sizeof(T))   // dx of the strip's rows, dy of the tile's columns
+            + (contract_blocked<T, C>() ? 7 * 8 * 4 + 32 * 8 * 4 : 0)  // dx rows' padding, second dy buffer (contract_block)
             + 3 * 8                                      // mbarriers
             + 127) / 128 * 128;
 }
@@ -1206,8 +1212,100 @@ __device__ __forceinline__ void contract_tile(const T* __restrict__ ring, int hb
     }
 }
 
+// 16 bytes from global to shared memory in the background (zeros unless `there`), and the wait for all
+// of this thread's.
+__device__ __forceinline__ void copy_row_async(void* dst, const void* src, bool there) {
+    const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(there ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void copy_rows_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Lanes that differ in `bit` share out two sums: those without it keep lo (and give hi away), those
+// with it keep hi.
+__device__ __forceinline__ float2 pass_half(float2 lo, float2 hi, int lane, int bit) {
+    const bool up = (lane & bit) != 0;
+    float2 keep = up ? hi : lo;
+    const float2 give = up ? lo : hi;
+    keep.x += __shfl_xor_sync(kFull, give.x, bit);
+    keep.y += __shfl_xor_sync(kFull, give.y, bit);
+    return keep;
+}
+
+// The same tile for C = 8 in FP32, a block of 8 rows x 4 columns per lane: lane 8 g + p takes rows
+// 4 g + i + 16 h (i < 4, h < 2) and columns p + 8 k (k < 4).  Each dk/dM is read once (a load's 32
+// banks are 8 g + p plus a constant) and serves both sums, against 4 dy rows kept in registers and a dx
+// row read per 4 cells, where a lane that walks a row and then a column reads two values of dk/dM and
+// four 16-byte vectors per cell.  xa holds the lane's row sums over a strip; the tile's column sums are
+// added up over the four lanes that share a column and end with lane q holding column q.
+// dx row r lies at xs + 8 r + 8 (r / 4), so that the four rows read at once lie in different banks.
+// What bounds it is latency at 12 warps per SM (168 registers, 71 KB a block: issue 37%, waits for
+// shared memory and the copies) and the work around the products: of about 1080 instructions a tile,
+// 256 are the two-wide FMAs.  48 x 48 pairs of 128 x 128 cells, d = 8: 0.109 -> 0.095 ms, 1.7 TB/s of
+// dk/dM.  The next tile's dy rows are copied to shared memory in the background; held in registers they
+// spilled 232 bytes.
+template <bool FULL, bool WRAP>
+__device__ __forceinline__ void contract_block(const float* __restrict__ ring, int hb, int coff, const float* __restrict__ xs,
+                                               const float* __restrict__ ys, int nr, int nc, int lane, float2 (&xa)[8][4],
+                                               float2 (&col)[4]) {
+    const int g = lane >> 3, p = lane & 7;
+    float2 y[4][4], ya[4][4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float4* v = reinterpret_cast<const float4*>(ys + (p + 8 * k) * 8);
+        const float4 lo = v[0], hi = v[1];
+        y[k][0] = make_float2(lo.x, lo.y);
+        y[k][1] = make_float2(lo.z, lo.w);
+        y[k][2] = make_float2(hi.x, hi.y);
+        y[k][3] = make_float2(hi.z, hi.w);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) ya[k][c] = make_float2(0.f, 0.f);
+    }
+    const int row0 = hb + 4 * g + p, pos0 = 8 * g + p + coff;
+    const float* base = ring + (row0 << 5);
+#pragma unroll
+    for (int n = 0; n < 8; ++n) {
+        const int i = n & 3, dr = i + 16 * (n >> 2);  // row 4 g + dr
+        const float4* v = reinterpret_cast<const float4*>(xs + (4 * g + dr) * 8 + (g + dr / 4) * 8);
+        const float4 lo = v[0], hi = v[1];
+        const float2 x[4] = {make_float2(lo.x, lo.y), make_float2(lo.z, lo.w), make_float2(hi.x, hi.y), make_float2(hi.z, hi.w)};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int u = dr + 8 * k;  // cell (row, column) at ring row row0 + u (mod 96)
+            int at = u * 32 + ((pos0 + 2 * i + 8 * k) & 31);
+            if (WRAP) at -= row0 + u >= 96 ? 96 * 32 : 0;
+            float m = base[at];
+            if (!FULL) m = (4 * g + dr < nr && p + 8 * k < nc) ? m : 0.f;
+            const float2 m2 = make_float2(m, m);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                xa[n][c] = __ffma2_rn(m2, y[k][c], xa[n][c]);
+                ya[k][c] = __ffma2_rn(m2, x[c], ya[k][c]);
+            }
+        }
+    }
+    float2 half[2][4];
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) half[k][c] = pass_half(ya[k][c], ya[k + 2][c], lane, 16);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) col[c] = pass_half(half[0][c], half[1][c], lane, 8);
+}
+
+// The strip's row sums from the eight lanes that share a row: lane 8 g + p ends with row
+// contract_row(lane)'s in xa[0].
+__device__ __forceinline__ int contract_row(int lane) { return 4 * (lane >> 3) + (lane & 3) + 16 * ((lane >> 2) & 1); }
+__device__ __forceinline__ void contract_rows(float2 (&xa)[8][4], int lane) {
+#pragma unroll
+    for (int w = 4; w > 0; w >>= 1)
+#pragma unroll
+        for (int n = 0; n < w; ++n)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) xa[n][c] = pass_half(xa[n][c], xa[n + w][c], lane, w);
+}
+
 template <typename T, int C>
-__global__ void __launch_bounds__(kContractWarps * 32) bwd_contract_kernel(BwdParams B) {
+__global__ void __launch_bounds__(kContractWarps * 32, (contract_blocked<T, C>() ? 3 : 0)) bwd_contract_kernel(BwdParams B) {
     constexpr int HB = 32 * 32 * static_cast<int>(sizeof(T));  // bytes of one half
     constexpr int WIN = contract_window<T, C>();
     using V = typename Vec<T>::type;
@@ -1223,8 +1321,10 @@ __global__ void __launch_bounds__(kContractWarps * 32) bwd_contract_kernel(BwdPa
     unsigned char* wsm = csm + wib * contract_warp_bytes<T, C>();
     T* ring = reinterpret_cast<T*>(wsm);                                   // [96 rows][32], circular
     T* xs = reinterpret_cast<T*>(wsm + 3 * HB);                            // [32][C]
-    T* ys = xs + 32 * C;                                                   // [32][C]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(wsm + 3 * HB + 2 * 32 * C * sizeof(T));
+    constexpr bool kBlocked = contract_blocked<T, C>();
+    constexpr int kPad = kBlocked ? 7 * 8 : 0;
+    T* ys = xs + 32 * C + kPad;                                            // [32][C], twice when blocked
+    uint64_t* bars = reinterpret_cast<uint64_t*>(wsm + 3 * HB + ((kBlocked ? 3 : 2) * 32 * C + kPad) * sizeof(T));
     T* acc = reinterpret_cast<T*>(csm + kContractWarps * contract_warp_bytes<T, C>());  // [C][WIN]
     if (lane == 0) {
         for (int k = 0; k < 3; ++k) mbar_init(bars + k, 1);
@@ -1285,7 +1385,7 @@ __global__ void __launch_bounds__(kContractWarps * 32) bwd_contract_kernel(BwdPa
                     {
                         const int xi = min((s << 5) + lane, rows - 1) >> lam;
                         const V* xr = reinterpret_cast<const V*>(xbase + static_cast<int64_t>(xi) * dpad + c0);
-                        V* xd = reinterpret_cast<V*>(xs + lane * C);
+                        V* xd = reinterpret_cast<V*>(xs + lane * C + (kBlocked ? lane / 4 * 8 : 0));
 #pragma unroll
                         for (int k = 0; k < C / W; ++k) {
                             V v = {};
@@ -1295,6 +1395,24 @@ __global__ void __launch_bounds__(kContractWarps * 32) bwd_contract_kernel(BwdPa
                     }
                     ContractAcc<T, C> xa;
                     xa.zero();
+                    float2 xb[8][4];
+                    if constexpr (kBlocked) {
+#pragma unroll
+                        for (int n = 0; n < 8; ++n)
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) xb[n][c] = make_float2(0.f, 0.f);
+                    }
+                    auto fetch_dy = [&](int b) {  // the dy rows of tile b, zero beyond the columns and coordinates
+                        const int j = w0 + (b << 5) + lane;
+                        const T* src = ybase + static_cast<int64_t>(min(j, cols - 1) >> lam) * dpad + c0;
+                        T* dst = ys + (b & 1) * 32 * C + lane * C;
+#pragma unroll
+                        for (int k = 0; k < C; k += W) {
+                            const bool there = j < cols && c0 + k < dpad;
+                            copy_row_async(dst + k, there ? src + k : src, there);
+                        }
+                    };
+                    if constexpr (kBlocked) fetch_dy(0);
                     for (int b = 0; b < ntiles; ++b) {
                         // half b (slot b % 3) was awaited as the upper half of tile b - 1, except for b = 0
                         const int s0 = b % 3, s1 = (b + 1) % 3;
@@ -1302,8 +1420,12 @@ __global__ void __launch_bounds__(kContractWarps * 32) bwd_contract_kernel(BwdPa
                         if (!await_slot(s1)) { stuck = true; break; }
                         const int j0 = w0 + (b << 5);
                         const int nc = min(32, cols - j0);  // valid columns of the tile
-                        __syncwarp();  // the previous tile's readers of ys are done
-                        {
+                        if constexpr (kBlocked) {
+                            copy_rows_wait();
+                            __syncwarp();  // this tile's dy rows are there, the previous tile's readers are done
+                            if (b + 1 < ntiles) fetch_dy(b + 1);
+                        } else {
+                            __syncwarp();  // the previous tile's readers of ys are done
                             const int yi = min(j0 + lane, cols - 1) >> lam;
                             const V* yr = reinterpret_cast<const V*>(ybase + static_cast<int64_t>(yi) * dpad + c0);
                             V* yd = reinterpret_cast<V*>(ys + lane * C);
@@ -1313,13 +1435,21 @@ __global__ void __launch_bounds__(kContractWarps * 32) bwd_contract_kernel(BwdPa
                                 if (lane < nc && c0 + k * W < dpad) v = __ldg(yr + k);
                                 yd[k] = v;
                             }
+                            __syncwarp();
                         }
-                        __syncwarp();
                         ContractAcc<T, C> ya;
                         ya.zero();
                         const int coff = (s * period + j0) & 31;
                         // slots 0-1 and 1-2 are contiguous in the ring; only slots 2-0 wrap
-                        if (nr == 32 && nc == 32) {
+                        if constexpr (kBlocked) {
+                            const T* yt = ys + (b & 1) * 32 * C;
+                            if (nr == 32 && nc == 32) {
+                                if (s0 == 2) contract_block<true, true>(ring, s0 * 32, coff, xs, yt, nr, nc, lane, xb, ya.s);
+                                else contract_block<true, false>(ring, s0 * 32, coff, xs, yt, nr, nc, lane, xb, ya.s);
+                            } else {
+                                contract_block<false, true>(ring, s0 * 32, coff, xs, yt, nr, nc, lane, xb, ya.s);
+                            }
+                        } else if (nr == 32 && nc == 32) {
                             if (s0 == 2) contract_tile<T, C, true, true>(ring, s0 * 32, coff, xs, ys, nr, nc, lane, xa, ya);
                             else contract_tile<T, C, true, false>(ring, s0 * 32, coff, xs, ys, nr, nc, lane, xa, ya);
                         } else {
@@ -1344,8 +1474,15 @@ __global__ void __launch_bounds__(kContractWarps * 32) bwd_contract_kernel(BwdPa
                             pending |= 1u << s0;
                         }
                     }
-                    if (lane < nr) {  // this strip's rows are its own: straight to the gradients
-                        const int xi = ((s << 5) + lane) >> lam;
+                    int r = lane;  // the row whose sums this lane holds
+                    if constexpr (kBlocked) {
+                        contract_rows(xb, lane);
+                        r = contract_row(lane);
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) xa.s[c] = xb[0][c];
+                    }
+                    if (r < nr) {  // this strip's rows are its own: straight to the gradients
+                        const int xi = ((s << 5) + r) >> lam;
 #pragma unroll
                         for (int c = 0; c < C; ++c) {
                             const T v = xa.get(c);
@@ -1365,6 +1502,7 @@ __global__ void __launch_bounds__(kContractWarps * 32) bwd_contract_kernel(BwdPa
         }
     }
     if (stuck) {  // the device error word is set; wait (bounded) for this warp's copies in flight
+        if constexpr (kBlocked) copy_rows_wait();
         for (int k = 0; k < 3; ++k)
             if (pending & (1u << k)) mbar_wait(bars + k, (parity >> k) & 1u);
     }
