@@ -1,7 +1,8 @@
 """GPU tests of the strip chain (a warp per strip, sk_chain.cuh) against one warp per pair.
 
 Both run the same cells in the same order, with M formed in the same order, so values are equal bit
-for bit; gradients differ only by the order of their FP64 atomics.  Shapes at the edges: rows that
+for bit; gradients differ only by the order of the contraction's atomics (FP64 sums, and in FP32
+its shared column sums too).  Shapes at the edges: rows that
 fill or just exceed a strip, fewer columns than a batch or a tile of M, wide and narrow increments,
 refinement, orders whose hand-off column takes 2 to 17 units, ragged sets, and hand-off buffers too
 few to hold every pair at once (a smaller workspace: pairs in groups, buffers used in turn).
