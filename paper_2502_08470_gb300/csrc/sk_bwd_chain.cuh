@@ -167,7 +167,6 @@ __global__ void __launch_bounds__(kFwdWarps * 32, (bwd_tape_min_blocks<T, N, INT
             const int c31 = cols + 30 - t;  // place of lane 31's column in the hand-off
             if (ends.in != nullptr && c31 < cols) {
                 if ((c31 & (Col::kCols - 1)) == 0) ends.take(c31 / Col::kCols, 0);
-                ends.ahead(c31);
                 uint32_t w[Col::kWords];
                 chain_words_load<kW>(ends.column(c31), w);
 #pragma unroll

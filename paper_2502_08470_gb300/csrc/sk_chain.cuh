@@ -20,8 +20,8 @@
 // (which cannot tear), so a word that shows the right tag is itself the data: no fence and no flag
 // to order.  (The ring of blocks that this replaced published progress with release stores and read
 // it with acquires, 3.0 us a step.)  The buffers are cleared before a launch, so no tag of an earlier
-// call is taken for one of this call's.  The consumer reads kCols columns at a time, ahead of
-// their use, into a small buffer in shared memory; the producer gathers as many there before it
+// call is taken for one of this call's.  The consumer reads kCols columns at a time, one batch ahead
+// of their use, into a small buffer in shared memory; the producer gathers as many there before it
 // writes them.
 //
 // Buffers.  A pair has a buffer for each strip that hands on, or ch_ring of them used in turn
@@ -123,11 +123,6 @@ template <int W>
 struct ChainEnds {
     using Col = ChainCol<W>;
     static constexpr int kLive = Col::kCols * Col::kUnits;  // lanes that carry a unit of a batch
-    // Columns by which a batch is read before its first is used.  Two (about the latency of L2) cost an
-    // eight-column strip less lag than a whole batch: one pair of 16384 x 16384 cells, order 6, 20.4 ->
-    // 19.6 ms; three 19.8, four and five a little more.  A batch of four or fewer is read when the one
-    // before it is taken: 64 pairs of 1024 x 1024 cells, interpolation N = 8, 3.65 ms, 3.72 with two.
-    static constexpr int kAhead = Col::kCols == 8 ? 2 : Col::kCols;
     const ChainUnit* in;   // the producer's buffer (NULL: no strip before this one)
     ChainUnit* out;        // this ticket's buffer (NULL: no strip after this one)
     uint32_t tag_in, tag_out;
@@ -173,15 +168,8 @@ struct ChainEnds {
                           (word % 2 ? w.y : w.x) != 0u;
         const bool any = __any_sync(kFull, mine) != 0;
         __syncwarp();
-        if constexpr (kAhead == Col::kCols) read_ahead(batch + 1);
+        read_ahead(batch + 1);
         return any;
-    }
-    // Called at every column c that the strip uses: reads the batch after c's, kAhead columns before its
-    // first is used.
-    __device__ __forceinline__ void ahead(int c) {
-        if constexpr (kAhead < Col::kCols) {
-            if ((c & (Col::kCols - 1)) == Col::kCols - kAhead) read_ahead(c / Col::kCols + 1);
-        }
     }
     __device__ __forceinline__ const uint32_t* column(int c) const {
         return fifo + (c & (2 * Col::kCols - 1)) * Col::kWords;
@@ -215,8 +203,8 @@ __host__ __device__ constexpr int chain_units(int N) {
     return (chain_words<T>(N) + 1) / 2;
 }
 
-// Steps by which a strip starts after the one below it: 31 for the wavefront, up to two batches of
-// columns and the latency of the hand-off.
+// Steps by which a strip starts after the one below it: 31 for the wavefront, two batches of columns
+// and the latency of the hand-off.
 constexpr int kChainLag = 50;
 
 struct ChainTicket {

@@ -4,7 +4,7 @@
 //
 // What bounds it: few pairs leave few warps on the GPU, so a step's latency counts, not its issue
 // slots.  Everything that a step waits for from outside the warp is therefore read ahead: the
-// incoming edges, a batch of columns at a time (ChainEnds), and M, in FP32, from a ring in shared
+// incoming edges a batch of columns earlier (ChainEnds), and M, in FP32, from a ring in shared
 // memory that the warp fills itself, two rows of the next 16 columns a step, beside the cell's own
 // chain of multiply-adds (MTile).  And what almost never happens is asked once for the warp, not
 // branched on per lane: exponents that differ (`mixed`), an M beyond tau (`big`).
@@ -131,7 +131,6 @@ __device__ __forceinline__ void sweep_strip(const Launch& L, int64_t item, const
         const int jj = t - lane;
         const bool active = static_cast<unsigned>(jj) < static_cast<unsigned>(cols) && in_grid;
         if (ends.in != nullptr) {  // lane 0 takes the edge that the strip before handed on
-            ends.ahead(t);
             uint32_t w[Col::kWords];
             chain_words_load<kW>(ends.column(t), w);
 #pragma unroll
