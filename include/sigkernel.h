@@ -393,7 +393,9 @@ float sigkernel_last_kernel_ms(void);
  * followed by a 32 to 64 ns sleep; a strip of a chain polls as often again for every strip before
  * it) before it gives up: the warp then records
  * SK_ERR_DEVICE_TIMEOUT in the device error word, finishes its sweep without waiting (that pair's
- * result is then wrong) and the kernel returns normally.  0 restores the default, 2^20 polls.
+ * result is then wrong) and the kernel returns normally.  A chained strip's wait for buffers polls as
+ * often for every 256 columns of the longest Y path, and again as long as strips of the call finish.
+ * 0 restores the default, 2^20 polls.
  * Process-wide; calls launched after it use the new limit.  The paper has no counterpart: this
  * is a robustness facility (a caller that wants a stalled pipeline reported sooner, and the test
  * of the timeout path).

@@ -320,6 +320,7 @@ struct ChainPlan {
     int units, ring, nb, groups;
     int64_t cap;      // tickets at most
     int64_t all;      // 16-byte units of the hand-off buffers
+    int cols;         // columns of the longest Y path
     size_t off_counts, counts_bytes, off_base, off_group, off_tickets, off_hand;
 };
 
@@ -392,7 +393,8 @@ bool plan_chain(ChainPlan& c, size_t& off, int64_t npairs, int64_t strips, int64
     c.nb = static_cast<int>(nb);
     c.groups = static_cast<int>(groups);
     c.all = groups > 1 ? budget / 2 * 2 : bound;
-    // cleared before each launch: used, total, gsize and gdone, strips done per item, histogram
+    c.cols = static_cast<int>(cols);
+    // cleared before each launch: used, total, finished, gsize and gdone, strips done per item, histogram
     c.off_counts = off;
     c.counts_bytes = align256(16 + (2 * static_cast<size_t>(groups) + static_cast<size_t>(npairs) + static_cast<size_t>(nb * groups)) * 4);
     off += c.counts_bytes;
@@ -871,6 +873,8 @@ int launch_chain_tickets(const ChainPlan& c, Launch& L, bool sorted, char* base,
     L.ch_done = done;
     L.ch_gsize = B.gsize;
     L.ch_gdone = gdone;
+    L.ch_finished = reinterpret_cast<int*>(counts + 12);
+    L.ch_cols = c.cols;
     L.order = nullptr;
     SK_CUDA(cudaMemsetAsync(counts, 0, c.counts_bytes, st));
     const int sb = static_cast<int>(std::min<int64_t>((L.npairs + 255) / 256, 4096));

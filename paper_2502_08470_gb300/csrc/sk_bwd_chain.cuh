@@ -106,10 +106,8 @@ __global__ void __launch_bounds__(kFwdWarps * 32, (bwd_tape_min_blocks<T, N, INT
                 bulk_load(ring + sl * kStepBytes, tape + static_cast<int64_t>(t) * kStepBytes, kStepBytes, bars + sl);
             }
         }
-        if (q + 1 < nstrips) {
-            if (!chain_claim(L, tk, ends.polls)) ends.stuck = true;
-            ends.out = chain_buffer(L, tk, q, cols, Col::kUnits);
-        }
+        if (!chain_claim(L, tk, q + 1 < nstrips)) ends.stuck = true;
+        else if (q + 1 < nstrips) ends.out = chain_buffer(L, tk, q, cols, Col::kUnits);
         ends.open();
         int stuck_step = -1;
         for (int t = nsteps - 1; t >= 0; --t) {

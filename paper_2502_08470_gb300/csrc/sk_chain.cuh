@@ -29,6 +29,14 @@
 // the workspace, pairs are put into groups, largest first, each of which fits half of it; a group's
 // tickets come after the group before's, and wait until the group that used their half is done
 // (ch_gdone).
+//
+// Bounds of the waits.  A wait for a column ends after a number of polls, since the strip before it is
+// at work (its own wait for buffers is over, chain_claim).  A wait for buffers can last as long as a
+// whole group's sweep, or several groups' in turn; it goes on as long as strips of the launch finish
+// (ch_finished) and ends after a stretch without any, as long as one strip's sweep may take
+// (chain_claim_polls).  Of the tickets not done, the first in the order waits for nothing that is not
+// done, so one finishes in every such stretch.  A ticket whose wait for buffers ran out hands nothing on:
+// the memory still belongs to others.
 #pragma once
 
 #include "sk_common.cuh"
@@ -240,14 +248,43 @@ __device__ __forceinline__ ChainUnit* chain_buffer(const Launch& L, const ChainT
     return L.ch_hand + L.ch_base[c.item] + (strip % L.ch_ring) * stride;
 }
 
-// Waits (bounded) until the ticket may write into its buffer.  Warp-uniform.
-__device__ __forceinline__ bool chain_claim(const Launch& L, const ChainTicket& c, uint32_t polls) {
+// A wait for finished strips (*p >= need): over when no strip of the launch has finished during `polls`
+// polls; false (and the device error word set) then.
+__device__ __forceinline__ bool chain_wait(const Launch& L, const int* p, int need, uint32_t polls) {
+    int seen = acquire_gpu(L.ch_finished);
+    for (;;) {
+        for (uint32_t it = 0; it < polls; ++it) {
+            if (acquire_gpu(p) >= need) return true;
+            __nanosleep(64);
+        }
+        const int now = acquire_gpu(L.ch_finished);
+        if (now == seen) break;
+        seen = now;
+    }
+    record_error(SK_ERR_DEVICE_TIMEOUT);
+    return false;
+}
+
+// Polls of one stretch of such a wait.  A poll takes 0.5 us or more, so the default limit gives each of
+// kChainWaitSteps steps of a sweep 2 ms, where the slowest (FP64 interpolation of the highest order, four
+// warps to a quarter of an SM) takes about 0.2 ms.
+constexpr int kChainWaitSteps = 256;
+__device__ __forceinline__ uint32_t chain_claim_polls(const Launch& L) {
+    const unsigned long long p = static_cast<unsigned long long>(wait_polls(L)) * (1 + (L.ch_cols + 31) / kChainWaitSteps);
+    return p > 0xfffffff0ull ? 0xfffffff0u : static_cast<uint32_t>(p);
+}
+
+// Waits until the buffer that the ticket writes is free and the strip before it has passed the same wait
+// (so that a wait for that strip's columns is a wait for a strip at work).  hands_on: a strip comes after
+// this one.  False when the wait ran out: the ticket must not write then.  Warp-uniform.
+__device__ __forceinline__ bool chain_claim(const Launch& L, const ChainTicket& c, bool hands_on) {
     bool ok = true;
     if ((threadIdx.x & 31) == 0) {
-        if (c.strip >= L.ch_ring) ok = wait_progress_gpu(L.ch_done + c.item, c.strip - L.ch_ring + 2, polls);
-        if (ok && c.group >= 2)
-            ok = wait_progress_gpu(reinterpret_cast<const int*>(L.ch_gdone) + c.group - 2,
-                                   static_cast<int>(L.ch_gsize[c.group - 2]), polls);
+        const uint32_t polls = chain_claim_polls(L);
+        if (c.group >= 2)
+            ok = chain_wait(L, reinterpret_cast<const int*>(L.ch_gdone) + c.group - 2, static_cast<int>(L.ch_gsize[c.group - 2]), polls);
+        const int writer = hands_on ? c.strip : c.strip - 1;
+        if (ok && writer >= L.ch_ring) ok = chain_wait(L, L.ch_done + c.item, writer - L.ch_ring + 2, polls);
     }
     return __shfl_sync(kFull, ok ? 1 : 0, 0) != 0;
 }
@@ -258,9 +295,10 @@ __device__ __forceinline__ void chain_finish(const Launch& L, const ChainTicket&
     __threadfence();
     atomicMax(L.ch_done + c.item, c.strip + 1);
     if (L.ch_groups > 1) atomicAdd(L.ch_gdone + c.group, 1u);
+    atomicAdd(L.ch_finished, 1);
 }
 
-// Polls for a strip's first wait: every strip before it may use up its own.
+// Polls of a wait for a column: every strip before this one may use up its own.
 __device__ __forceinline__ uint32_t chain_polls(const Launch& L, int strip) {
     const unsigned long long p = static_cast<unsigned long long>(wait_polls(L)) * static_cast<unsigned long long>(strip + 1);
     return p > 0xfffffff0ull ? 0xfffffff0u : static_cast<uint32_t>(p);

@@ -182,8 +182,9 @@ struct Launch {
     int64_t mx_stride;
     // Strip chain (sk_chain.cuh): the tickets in order, (work item, strip, ticket of the strip before
     // + 1, group), and how many there are; the hand-off buffers, each item's first unit in them and
-    // the buffers an item uses in turn; strips done per item; and, with more than one group, the
-    // tickets of each and how many are done.  Counters are cleared before the launch.
+    // the buffers an item uses in turn; strips done per item; with more than one group, the tickets of
+    // each and how many are done; tickets done in all, and the columns of the longest Y path (they bound
+    // the waits for buffers).  Counters are cleared before the launch.
     const int4* ch_tickets;
     const unsigned int* ch_total;
     ChainUnit* ch_hand;
@@ -193,6 +194,8 @@ struct Launch {
     int* ch_done;
     const unsigned int* ch_gsize;
     unsigned int* ch_gdone;
+    int* ch_finished;
+    int32_t ch_cols;
 };
 
 // Width, in elements of T, of one lane's tape row.
@@ -315,18 +318,12 @@ __device__ __forceinline__ bool wait_progress(const int* p, int need, uint32_t p
     return false;
 }
 
-// A counter in global memory, read with acquire at GPU scope (the strip chain's buffers): accesses
-// after the wait come after those that its writer's fence ordered before the count.
-// Bounded wait for *p >= need; false (and the device error word set) when it runs out.
-__device__ __forceinline__ bool wait_progress_gpu(const int* p, int need, uint32_t polls) {
-    for (uint32_t it = 0; it < polls; ++it) {
-        int v;
-        asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-        if (v >= need) return true;
-        __nanosleep(64);
-    }
-    record_error(SK_ERR_DEVICE_TIMEOUT);
-    return false;
+// A counter in global memory, read with acquire at GPU scope: accesses after it come after those that
+// its writer's fence ordered before the count.
+__device__ __forceinline__ int acquire_gpu(const int* p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
 }
 
 // Pop the next work item for a warp (lane 0 takes it, all lanes receive it).

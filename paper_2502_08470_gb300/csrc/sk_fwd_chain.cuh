@@ -305,10 +305,8 @@ __global__ void __launch_bounds__(kFwdWarps * 32, (fwd_chain_min_blocks<T, N, NE
         ends.next = ChainUnit{0ull, 0ull};
         ends.in = g > 0 ? chain_buffer(L, tk, g - 1, ends.cols, Ends::Col::kUnits) : nullptr;
         ends.out = nullptr;
-        if (g + 1 < nstrips) {
-            if (!chain_claim(L, tk, ends.polls)) ends.stuck = true;
-            ends.out = chain_buffer(L, tk, g, ends.cols, Ends::Col::kUnits);
-        }
+        if (!chain_claim(L, tk, g + 1 < nstrips)) ends.stuck = true;
+        else if (g + 1 < nstrips) ends.out = chain_buffer(L, tk, g, ends.cols, Ends::Col::kUnits);
         ends.open();
         sweep_strip<T, N, NE, INTERP, DMT>(L, tk.item, P, g, ends, xs, mring);
         __syncwarp();  // every lane is done with the incoming buffer
