@@ -839,8 +839,13 @@ int plan_forward_within(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t
     int rc = plan_forward(X, Y, d, dtype, o, mode, npairs, p, !tape, tape);
     if (rc != SK_OK || p.total <= bytes || !p.chain.on) return rc;
     const size_t rest = p.total - align256(static_cast<size_t>(p.chain.all) * 16);
-    if ((rc = plan_forward(X, Y, d, dtype, o, mode, npairs, p, !tape, tape, bytes > rest ? bytes - rest : 0)) != SK_OK) return rc;
-    if (p.total <= bytes || !p.chain.on) return rc;
+    size_t limit = bytes > rest ? bytes - rest : 0;
+    // (more groups take more counters, so the buffers may have to shrink again)
+    for (int tries = 0; tries < 4 && limit > 0; ++tries) {
+        if ((rc = plan_forward(X, Y, d, dtype, o, mode, npairs, p, !tape, tape, limit)) != SK_OK) return rc;
+        if (p.total <= bytes || !p.chain.on) return rc;
+        limit -= std::min(limit, p.total - bytes);
+    }
     return plan_forward(X, Y, d, dtype, o, mode, npairs, p, !tape, tape, 0);
 }
 

@@ -1,5 +1,6 @@
 """GPU tests of the strip chain where its buffers do not hold everything at once: a pair whose strips use
-fewer buffers than it has hand-offs in turn; and two calls at once on two streams.
+fewer buffers than it has hand-offs in turn, and pairs in several groups that take the two halves of the
+buffers in turn, with waits that last longer than the limit on polls; and two calls at once on two streams.
 
 A workspace smaller than the plan's leaves fewer buffers; that the chain still runs in it (and not one
 warp per pair) shows in a limit of one poll, which only a chain's waits can exhaust.  The same cells
@@ -50,6 +51,28 @@ def test_buffers_used_in_turn(compute, N, drop):
     ws = torch.empty(full - drop * 304 * _units(N, compute) * 16, dtype=torch.uint8, device="cuda")
     assert sk.device_status() == 0
     got = sk.sigkernel_gram(X, Y, strip_pipeline=True, workspace=ws, **kw)
+    assert sk.device_status() == 0
+    assert torch.equal(got, sk.sigkernel_gram(X, Y, strip_pipeline=False, **kw))
+    assert _chained(X, Y, ws, kw)
+
+
+@pytest.mark.parametrize("scheme,N,compute,limit", [("interp", 12, "f64", 1 << 15), ("approx", 6, "f32", 0)])
+def test_groups(scheme, N, compute, limit):
+    """Nine pairs of 14 strips, one to each half of the buffers: nine groups.  With the slow FP64 steps a
+    pair takes about 50 ms and the limit's polls about 20, so the wait of a group's first strip for the
+    group before the last goes on only because strips finish meanwhile."""
+    X, Y = _paths(3, 430, 2, 703), _paths(3, 301, 2, 704)
+    kw = dict(scheme=scheme, degree=N, compute=compute, tensor_cores=False)
+    full = sk.gram_workspace(X, Y, scheme=scheme, degree=N, compute=compute, strip_pipeline=True).numel()
+    pair = 13 * 304 * _units(N, compute) * 16  # hand-off bytes of a pair
+    ws = torch.empty(full - 9 * pair + 2 * pair + pair // 2, dtype=torch.uint8, device="cuda")
+    assert sk.device_status() == 0
+    sk.set_wait_limit(limit)
+    try:
+        got = sk.sigkernel_gram(X, Y, strip_pipeline=True, workspace=ws, **kw)
+        torch.cuda.synchronize()
+    finally:
+        sk.set_wait_limit(0)
     assert sk.device_status() == 0
     assert torch.equal(got, sk.sigkernel_gram(X, Y, strip_pipeline=False, **kw))
     assert _chained(X, Y, ws, kw)
