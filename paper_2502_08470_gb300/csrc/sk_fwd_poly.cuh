@@ -434,7 +434,11 @@ __device__ __forceinline__ void sweep_poly(const Launch& L, int64_t item, const 
 #pragma unroll
         for (int n = 0; n <= N; ++n) b[n] = __shfl_up_sync(kFull, bo[n], 1);
         int eb = kRescale ? __shfl_up_sync(kFull, eo, 1) : 0;
-        const bool active = static_cast<unsigned>(jj) < static_cast<unsigned>(cols) && row < rows;
+        // (row < rows says that the strip is one of the pair's.  Said twice in the plain sweep that reads its M,
+        // the compiler keeps order 6 at 64 registers, eight blocks per SM: 4864 pairs of 513 points, d = 8,
+        // in 11.2 ms instead of 13.8 at 72 registers, or 12.2 at 64 by a launch bound.)
+        const bool active = static_cast<unsigned>(jj) < static_cast<unsigned>(cols) && row < rows &&
+                            (!MX || DMT || g < nstrips);
         if (active && lane == 0) {
             if (g == 0) {  // q^{0,j} = e_0 (left boundary k(0, .) = 1)
 #pragma unroll
