@@ -1258,6 +1258,8 @@ struct TapeBwdPlan {
     TapePlan t;
     const void* kern;
     ChainPlan chain;     // a warp per strip instead of one per pair
+    int64_t resident;    // items resident at once with a warp each (whether chained or not): what a tape
+                         // chunk is measured against.  A chain's blocks count strips, not items.
     const void* ckern;
     int smem_bytes, cblocks, csmem, cC;
     int64_t cols_max, off_rbuf, off_rexp, slot_bytes, mb_stride, acc_bytes;
@@ -1340,6 +1342,7 @@ int plan_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t 
     b.tc_sms = sms;
     b.cblocks = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(npairs, static_cast<int64_t>(sms) * cper_sm)));
     int64_t want = (npairs + kFwdWarps - 1) / kFwdWarps;
+    b.resident = std::max<int64_t>(1, std::min(want, static_cast<int64_t>(sms) * per_sm)) * kFwdWarps;
     // too few pairs to fill the GPU with one warp each: a warp per strip, as in the forward
     b.chain = ChainPlan{};
     const void* chain_kern = fd ? nullptr : bwd_chain_ptr(p.T, o->degree, interp);
@@ -1654,7 +1657,7 @@ int plan_mmd2_blocks(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t d
         if ((rc = plan_tape(xs[k], ys[k], ok, p1.T, 1, t1)) != SK_OK) return rc;
         TapeBwdPlan whole;
         if ((rc = plan_backward_tape(xs[k], ys[k], d, dtype, ok, modes[k], m.items[k], whole)) != SK_OK) return rc;
-        const int64_t resident = std::max<int64_t>(1, static_cast<int64_t>(whole.f.blocks) * kFwdWarps);
+        const int64_t resident = whole.resident;
         int64_t c = std::max<int64_t>(1, static_cast<int64_t>(kTapeChunkBudget / std::max<size_t>(t1.stride, 1)));
         if (c < m.items[k] && c > resident) c -= c % resident;
         m.chunk[k] = std::min(c, m.items[k]);
@@ -1820,7 +1823,7 @@ int plan_backward_chunked(const sk_paths* X, const sk_paths* Y, int32_t d, int32
     if ((rc = plan_tape(X, Y, o, p1.T, 1, t1)) != SK_OK) return rc;
     TapeBwdPlan whole;
     if ((rc = plan_backward_tape(X, Y, d, dtype, o, mode, std::max<int64_t>(items, 1), whole)) != SK_OK) return rc;
-    const int64_t resident = std::max<int64_t>(1, static_cast<int64_t>(whole.f.blocks) * kFwdWarps);
+    const int64_t resident = whole.resident;
     int64_t chunk = std::max<int64_t>(1, static_cast<int64_t>(kTapeChunkBudget / std::max<size_t>(t1.stride, 1)));
     if (chunk < items && chunk > resident) chunk -= chunk % resident;
     chunk = std::max<int64_t>(1, std::min(chunk, items));
