@@ -1414,6 +1414,7 @@ int launch_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int32_
     L.dpad = p.dpad;
     L.inc_mode = inc_mode;
     L.lam = o->dyadic;
+    L.wait_limit = g_wait_limit.load(std::memory_order_relaxed);
     L.mode = mode;
     L.npairs = npairs;
     L.item_base = item_base;
