@@ -542,8 +542,8 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     // Launch shape.  Explicit requests (warps_per_block, the strip-pipeline flags) win; otherwise a
     // shape that sigkernel_autotune measured for this shape of call; otherwise the defaults.
     int wpb_req = 0, pipe_req = 0;  // pipe_req: 1 strip pipeline, -1 none, 0 the default rule
-    if (allow_coop) {
-        wpb_req = o->warps_per_block;
+    if (allow_coop) wpb_req = o->warps_per_block;
+    if (allow_coop || tape) {
         if (o->flags & SK_FLAG_STRIP_PIPELINE) pipe_req = 1;
         if (o->flags & SK_FLAG_NO_STRIP_PIPELINE) pipe_req = -1;
     }
