@@ -117,7 +117,7 @@ enum {
                                        bit for bit where M is formed the same way (see
                                        SK_FLAG_NO_TC).  A chain needs workspace for its hand-off (at
                                        most 8 GiB); in a smaller workspace the call uses fewer
-                                       buffers, or one warp per pair */
+                                       buffers, or one warp per pair (sigkernel_workspace_least) */
     SK_FLAG_NO_TILED_M = 128,       /* forward, polynomial schemes in FP32, where the tensor cores
                                        do not compute M (see SK_FLAG_NO_TC): form each cell's M
                                        from its two increment rows.  By default, with d > 8, each
@@ -185,6 +185,15 @@ enum { SK_OP_PAIRS = 0, SK_OP_GRAM = 1, SK_OP_BACKWARD = 2, SK_OP_MMD2 = 3, SK_O
  */
 int sigkernel_workspace_size(int32_t op, const sk_paths* X, const sk_paths* Y, int32_t d,
                              int64_t npairs, const sk_options* opt, size_t* bytes);
+
+/*
+ * sigkernel_workspace_least -- as sigkernel_workspace_size, the least workspace with which the call
+ * runs: without the buffers of strip chains (up to 8 GiB), and of the tensor-core M where a chain
+ * would have stood in its place.  The call takes any workspace from this size on and uses what of a
+ * chain fits; one that allocates its own takes this size when the device has no room for the other.
+ */
+int sigkernel_workspace_least(int32_t op, const sk_paths* X, const sk_paths* Y, int32_t d,
+                              int64_t npairs, const sk_options* opt, size_t* bytes);
 
 /*
  * sigkernel_pairs -- out[k] = k_hat(X_{pair_a[k]}, Y_{pair_b[k]}) for k < npairs.

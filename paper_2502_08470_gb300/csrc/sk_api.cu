@@ -86,6 +86,19 @@ struct OwnedWorkspace {
     ~OwnedWorkspace() {
         if (p) cudaFreeAsync(p, st);
     }
+    // Allocates `bytes` for the call; SK_ERR_WORKSPACE when the device has no room for them.
+    int take(void** ws, size_t bytes, cudaStream_t stream) {
+        const cudaError_t e = cudaMallocAsync(&p, bytes, stream);
+        if (e == cudaSuccess) {
+            *ws = p;
+            st = stream;
+            return SK_OK;
+        }
+        p = nullptr;
+        if (e != cudaErrorMemoryAllocation) return fail(SK_ERR_CUDA, "cudaMallocAsync: %s", cudaGetErrorString(e));
+        cudaGetLastError();
+        return fail(SK_ERR_WORKSPACE, "no device memory for a workspace of %zu bytes", bytes);
+    }
     cudaError_t release() {  // the success path's free, with its status
         void* q = p;
         p = nullptr;
@@ -495,7 +508,7 @@ bool chain_pays(const sk_paths* X, const sk_paths* Y, int64_t points, int lam, i
 // allow_coop: the caller launches p.kern itself with p.threads (the plain forward); adjoint
 // plans reuse this layout with their own one-warp-per-pair kernels and pass false.  tape: the
 // forward records a tape (one warp per pair; its own kernels for the approximation scheme).
-// chain_limit: bytes a strip chain's buffers may take (0: no chain).
+// chain_limit: bytes a strip chain's buffers may take (0: no chain).  Plans that are neither have none.
 constexpr size_t kChainAny = ~size_t(0);
 int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, const sk_options* o,
                  int mode, int64_t npairs, Plan& p, bool allow_coop = false, bool tape = false,
@@ -612,7 +625,7 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     }
     bool want_chain = false;
     const int64_t strips = (max_rows + 31) / 32;
-    if (poly && chain_limit > 0 && pipe_req >= 0 && strips >= 2 && npairs > 0) {
+    if (poly && (allow_coop || tape) && pipe_req >= 0 && strips >= 2 && npairs > 0) {
         want_chain = pipe_req > 0 || chain_pays(X, Y, points, lam, npairs, strips, max_cols,
                                                 static_cast<int64_t>(sms) * per_sm * kFwdWarps, p.T);
     }
@@ -650,7 +663,7 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     const int64_t mx_bytes = static_cast<int64_t>(align256(static_cast<size_t>((mx_steps + 3) / 4) * 32 * 16));
     const bool mx_scheme = p.T == 1 && o->scheme == SK_POLY_APPROX && p.dpad >= 8 && p.dpad <= 32 && !(o->flags & SK_FLAG_NO_TC);
     const int chain_u = p.T ? chain_units<float>(o->degree) : chain_units<double>(o->degree);
-    if (want_chain) {
+    if (want_chain && chain_limit > 0) {
         const void* ck = fwd_poly_kernel_ptr(p.T, o->scheme == SK_POLY_INTERP, o->degree, true, false, tape);
         size_t none = 0;
         if (ck && plan_chain(p.chain, none, npairs, strips, max_cols, chain_u, chain_limit)) {
@@ -665,7 +678,8 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
             }
         }
     }
-    if (!p.chain.on && mx_scheme) {
+    // (a call without room for a chain has none for the M of its long pairs either)
+    if (!p.chain.on && mx_scheme && !(want_chain && chain_limit == 0)) {
         const void* km = fwd_poly_kernel_ptr(p.T, false, o->degree, false, false, tape, true);
         if (km) {
             const int64_t stride = mx_bytes;
@@ -843,7 +857,8 @@ int plan_forward_within(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t
     // (more groups take more counters, so the buffers may have to shrink again)
     for (int tries = 0; tries < 4 && limit > 0; ++tries) {
         if ((rc = plan_forward(X, Y, d, dtype, o, mode, npairs, p, !tape, tape, limit)) != SK_OK) return rc;
-        if (p.total <= bytes || !p.chain.on) return rc;
+        if (p.total <= bytes) return rc;
+        if (!p.chain.on) break;
         limit -= std::min(limit, p.total - bytes);
     }
     return plan_forward(X, Y, d, dtype, o, mode, npairs, p, !tape, tape, 0);
@@ -925,9 +940,12 @@ int run_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     OwnedWorkspace owned;
     if (!ws) {
-        SK_CUDA(cudaMallocAsync(&ws, p.total, st));
-        owned.p = ws;
-        owned.st = st;
+        rc = owned.take(&ws, p.total, st);
+        if (rc == SK_ERR_WORKSPACE && p.chain.on) {  // no room for a chain's buffers
+            if ((rc = plan_forward(X, Y, d, dtype, o, mode, npairs, p, tape == nullptr, tape != nullptr, 0)) != SK_OK) return rc;
+            rc = owned.take(&ws, p.total, st);
+        }
+        if (rc != SK_OK) return rc;
     } else if (ws_bytes < p.total) {
         return fail(SK_ERR_WORKSPACE, "workspace %zu bytes < %zu required", ws_bytes, p.total);
     }
@@ -1228,9 +1246,7 @@ int run_backward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     OwnedWorkspace owned;
     if (!ws) {
-        SK_CUDA(cudaMallocAsync(&ws, b.total, st));
-        owned.p = ws;
-        owned.st = st;
+        if ((rc = owned.take(&ws, b.total, st)) != SK_OK) return rc;
     } else if (ws_bytes < b.total) {
         return fail(SK_ERR_WORKSPACE, "workspace %zu bytes < %zu required", ws_bytes, b.total);
     }
@@ -1503,9 +1519,12 @@ int run_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t d
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     OwnedWorkspace owned;
     if (!ws) {
-        SK_CUDA(cudaMallocAsync(&ws, b.total, st));
-        owned.p = ws;
-        owned.st = st;
+        rc = owned.take(&ws, b.total, st);
+        if (rc == SK_ERR_WORKSPACE && b.chain.on) {
+            if ((rc = plan_backward_tape(X, Y, d, dtype, o, mode, npairs, b, false)) != SK_OK) return rc;
+            rc = owned.take(&ws, b.total, st);
+        }
+        if (rc != SK_OK) return rc;
     } else if (ws_bytes < b.total) {
         return fail(SK_ERR_WORKSPACE, "workspace %zu bytes < %zu required", ws_bytes, b.total);
     }
@@ -1613,7 +1632,8 @@ struct MmdPlan {
 };
 
 int plan_mmd2_blocks(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t dtype, const sk_options* o, bool grads,
-                     bool pooled, MmdPlan& m) {
+                     bool pooled, MmdPlan& m, bool chain_ok) {
+    const size_t chain = chain_ok ? kChainAny : 0;
     if (!A || !Bp || !o) return fail(SK_ERR_INVALID_ARG, "NULL argument");
     if (A->count < 1 || Bp->count < 1) return fail(SK_ERR_INVALID_ARG, "MMD^2 needs non-empty path sets");
     const bool unb = (o->flags & SK_FLAG_UNBIASED) != 0;
@@ -1648,7 +1668,8 @@ int plan_mmd2_blocks(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t d
         const sk_options* ok = k < 2 ? &m.os : &m.of;
         if (!grads) {
             m.chunk[k] = m.items[k];
-            if ((rc = plan_forward(xs[k], ys[k], d, dtype, ok, modes[k], m.items[k], m.f[k], true)) != SK_OK) return rc;
+            if ((rc = plan_forward(xs[k], ys[k], d, dtype, ok, modes[k], m.items[k], m.f[k], true, false, chain)) != SK_OK)
+                return rc;
             m.sub = std::max(m.sub, m.f[k].total);
             continue;
         }
@@ -1669,17 +1690,24 @@ int plan_mmd2_blocks(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t d
                             "MMD^2 gradients of this scheme need forward tapes, and these paths are too long for a "
                             "tape chunk to fill the GPU");
             m.chunk[k] = m.items[k];
-            if ((rc = plan_forward(xs[k], ys[k], d, dtype, ok, modes[k], m.items[k], m.f[k], true)) != SK_OK) return rc;
+            if ((rc = plan_forward(xs[k], ys[k], d, dtype, ok, modes[k], m.items[k], m.f[k], true, false, chain)) != SK_OK)
+                return rc;
             if ((rc = plan_backward(xs[k], ys[k], d, dtype, ok, modes[k], m.items[k], m.cb[k])) != SK_OK) return rc;
             m.sub = std::max(m.sub, std::max(m.f[k].total, m.cb[k].total));
             continue;
         }
-        if ((rc = plan_forward(xs[k], ys[k], d, dtype, ok, modes[k], m.chunk[k], m.f[k], false, true)) != SK_OK)
+        if ((rc = plan_forward(xs[k], ys[k], d, dtype, ok, modes[k], m.chunk[k], m.f[k], false, true, chain)) != SK_OK)
             return rc;
-        if ((rc = plan_backward_tape(xs[k], ys[k], d, dtype, ok, modes[k], m.chunk[k], m.tb[k])) != SK_OK) return rc;
+        if ((rc = plan_backward_tape(xs[k], ys[k], d, dtype, ok, modes[k], m.chunk[k], m.tb[k], chain_ok)) != SK_OK) return rc;
         TapePlan tc;
         if ((rc = plan_tape(xs[k], ys[k], ok, p1.T, m.chunk[k], tc)) != SK_OK) return rc;
         m.tape_bytes = std::max(m.tape_bytes, tc.total);
+        if (m.items[k] % m.chunk[k]) {  // the last chunk's forward may be planned another way
+            Plan last;
+            if ((rc = plan_forward(xs[k], ys[k], d, dtype, ok, modes[k], m.items[k] % m.chunk[k], last, false, true, chain)) != SK_OK)
+                return rc;
+            m.sub = std::max(m.sub, last.total);
+        }
         m.sub = std::max(m.sub, std::max(m.f[k].total, m.tb[k].total));
     }
     const int64_t na = A->count, nb = Bp->count;
@@ -1694,15 +1722,16 @@ int plan_mmd2_blocks(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t d
     return SK_OK;
 }
 
+// chain_ok: strip chains, whose buffers may take much more than the rest, may be used.
 int plan_mmd2(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t dtype, const sk_options* o, bool grads,
-              MmdPlan& m) {
+              MmdPlan& m, bool chain_ok = true) {
     if (A && Bp && A->count > 0 && Bp->count > 0 &&
         4 * std::max(A->max_len, Bp->max_len) <= 5 * std::min(A->max_len, Bp->max_len)) {
         // (a pooled block that does not fit a plan, or whose tape chunks cannot fill the GPU, falls back)
-        if (plan_mmd2_blocks(A, Bp, d, dtype, o, grads, true, m) == SK_OK && (!grads || m.tape[0])) return SK_OK;
+        if (plan_mmd2_blocks(A, Bp, d, dtype, o, grads, true, m, chain_ok) == SK_OK && (!grads || m.tape[0])) return SK_OK;
         t_last_error.clear();
     }
-    return plan_mmd2_blocks(A, Bp, d, dtype, o, grads, false, m);
+    return plan_mmd2_blocks(A, Bp, d, dtype, o, grads, false, m, chain_ok);
 }
 
 int run_mmd2(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t dtype, const sk_options* o, double* out,
@@ -1715,10 +1744,14 @@ int run_mmd2(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t dtype, co
     const bool unb = (o->flags & SK_FLAG_UNBIASED) != 0;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     OwnedWorkspace owned;
+    if (ws && ws_bytes < m.total && (rc = plan_mmd2(A, Bp, d, dtype, o, grads, m, false)) != SK_OK) return rc;
     if (!ws) {
-        SK_CUDA(cudaMallocAsync(&ws, m.total, st));
-        owned.p = ws;
-        owned.st = st;
+        rc = owned.take(&ws, m.total, st);
+        if (rc == SK_ERR_WORKSPACE) {
+            if ((rc = plan_mmd2(A, Bp, d, dtype, o, grads, m, false)) != SK_OK) return rc;
+            rc = owned.take(&ws, m.total, st);
+        }
+        if (rc != SK_OK) return rc;
     } else if (ws_bytes < m.total) {
         return fail(SK_ERR_WORKSPACE, "workspace %zu bytes < %zu required", ws_bytes, m.total);
     }
@@ -1816,7 +1849,7 @@ struct ChunkBwdPlan {
 };
 
 int plan_backward_chunked(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, const sk_options* o,
-                          int mode, int64_t items, ChunkBwdPlan& c) {
+                          int mode, int64_t items, ChunkBwdPlan& c, bool chain_ok = true) {
     Plan p1;
     int rc;
     if ((rc = plan_forward(X, Y, d, dtype, o, mode, 1, p1)) != SK_OK) return rc;
@@ -1837,8 +1870,8 @@ int plan_backward_chunked(const sk_paths* X, const sk_paths* Y, int32_t d, int32
     }
     c.items = items;
     c.chunk = chunk;
-    if ((rc = plan_forward(X, Y, d, dtype, o, mode, chunk, c.f, false, true)) != SK_OK) return rc;
-    if ((rc = plan_backward_tape(X, Y, d, dtype, o, mode, chunk, c.tb)) != SK_OK) return rc;
+    if ((rc = plan_forward(X, Y, d, dtype, o, mode, chunk, c.f, false, true, chain_ok ? kChainAny : 0)) != SK_OK) return rc;
+    if ((rc = plan_backward_tape(X, Y, d, dtype, o, mode, chunk, c.tb, chain_ok)) != SK_OK) return rc;
     TapePlan tc;
     if ((rc = plan_tape(X, Y, o, p1.T, chunk, tc)) != SK_OK) return rc;
     c.tape_bytes = tc.total;
@@ -1847,6 +1880,11 @@ int plan_backward_chunked(const sk_paths* X, const sk_paths* Y, int32_t d, int32
     c.ginc_a = align256(static_cast<size_t>(X->rows_total) * p1.dpad * sizeof(double));
     c.ginc_bytes = c.ginc_a + (p1.same_xy ? 0 : align256(static_cast<size_t>(Y->rows_total) * p1.dpad * sizeof(double)));
     c.sub = std::max(c.f.total, c.tb.total);
+    if (items > chunk && items % chunk) {  // the last chunk's forward may be planned another way
+        Plan last;
+        if ((rc = plan_forward(X, Y, d, dtype, o, mode, items % chunk, last, false, true, chain_ok ? kChainAny : 0)) != SK_OK) return rc;
+        c.sub = std::max(c.sub, last.total);
+    }
     c.total = c.ginc_bytes + align256(c.tape_bytes) + c.out_bytes + c.sub + 512;
     return SK_OK;
 }
@@ -1876,10 +1914,14 @@ int run_backward_chunked(const sk_paths* X, const sk_paths* Y, int32_t d, int32_
     if (!gout) return fail(SK_ERR_INVALID_ARG, "grad_out is NULL");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     OwnedWorkspace owned;
+    if (ws && ws_bytes < c.total && (rc = plan_backward_chunked(X, Y, d, dtype, o, mode, npairs, c, false)) != SK_OK) return rc;
     if (!ws) {
-        SK_CUDA(cudaMallocAsync(&ws, c.total, st));
-        owned.p = ws;
-        owned.st = st;
+        rc = owned.take(&ws, c.total, st);
+        if (rc == SK_ERR_WORKSPACE) {
+            if ((rc = plan_backward_chunked(X, Y, d, dtype, o, mode, npairs, c, false)) != SK_OK) return rc;
+            rc = owned.take(&ws, c.total, st);
+        }
+        if (rc != SK_OK) return rc;
     } else if (ws_bytes < c.total) {
         return fail(SK_ERR_WORKSPACE, "workspace %zu bytes < %zu required", ws_bytes, c.total);
     }
@@ -1924,9 +1966,9 @@ struct MmdTestPlan {
 };
 
 int plan_mmd2_test(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t dtype, const sk_options* o, int64_t nperm,
-                   MmdTestPlan& t) {
+                   MmdTestPlan& t, bool chain_ok = true) {
     if (nperm < 0 || nperm > kMaxPerm) return fail(SK_ERR_INVALID_ARG, "nperm %lld outside [0, 2^24]", (long long)nperm);
-    int rc = plan_mmd2(A, Bp, d, dtype, o, false, t.m);
+    int rc = plan_mmd2(A, Bp, d, dtype, o, false, t.m, chain_ok);
     if (rc != SK_OK) return rc;
     const int64_t n = A->count + Bp->count;
     if (n > kMaxPooled) return fail(SK_ERR_UNSUPPORTED, "%lld pooled paths (this build: <= %lld)", (long long)n,
@@ -1946,10 +1988,14 @@ int run_mmd2_test(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t dtyp
     if (rc != SK_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     OwnedWorkspace owned;
+    if (ws && ws_bytes < t.total && (rc = plan_mmd2_test(A, Bp, d, dtype, o, nperm, t, false)) != SK_OK) return rc;
     if (!ws) {
-        SK_CUDA(cudaMallocAsync(&ws, t.total, st));
-        owned.p = ws;
-        owned.st = st;
+        rc = owned.take(&ws, t.total, st);
+        if (rc == SK_ERR_WORKSPACE) {
+            if ((rc = plan_mmd2_test(A, Bp, d, dtype, o, nperm, t, false)) != SK_OK) return rc;
+            rc = owned.take(&ws, t.total, st);
+        }
+        if (rc != SK_OK) return rc;
     } else if (ws_bytes < t.total) {
         return fail(SK_ERR_WORKSPACE, "workspace %zu bytes < %zu required", ws_bytes, t.total);
     }
@@ -1974,6 +2020,82 @@ int run_mmd2_test(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t dtyp
     SK_CUDA(launch_mmd_perm(K, n, na, labels, nperm, (o->flags & SK_FLAG_UNBIASED) ? 1 : 0, scratch, out, st));
     SK_CUDA(owned.release());
     return SK_OK;
+}
+
+// sigkernel_workspace_size (chain_ok) and sigkernel_workspace_least.
+int workspace(int32_t op, const sk_paths* X, const sk_paths* Y, int32_t d, int64_t npairs, const sk_options* opt,
+              bool chain_ok, size_t* bytes) {
+    t_last_error.clear();
+    if (!bytes) return fail(SK_ERR_INVALID_ARG, "bytes is NULL");
+    *bytes = 0;
+    if (!opt || !X || !Y) return fail(SK_ERR_INVALID_ARG, "NULL argument");
+    Plan p;
+    int rc;
+    const int dtype = SK_F64;  // sizes do not depend on the input element type
+    const size_t chain = chain_ok ? kChainAny : 0;
+    switch (op) {
+        case SK_OP_PAIRS:
+            rc = plan_forward(X, Y, d, dtype, opt, kPairsList, npairs, p, true, false, chain);
+            break;
+        case SK_OP_GRAM: {
+            bool sym = (opt->flags & SK_FLAG_SYMMETRIC) != 0;
+            rc = plan_forward(X, Y, d, dtype, opt, sym ? kGramUpper : kGramFull, gram_items(X, Y, sym), p, true,
+                              false, chain);
+            break;
+        }
+        case SK_OP_BACKWARD: {
+            const bool gram = npairs < 0;
+            const bool sym = gram && (opt->flags & SK_FLAG_SYMMETRIC);
+            if (uses_tape_chunks(opt)) {
+                ChunkBwdPlan c;
+                rc = plan_backward_chunked(X, Y, d, dtype, opt, gram ? (sym ? kGramUpper : kGramFull) : kPairsList,
+                                           gram ? gram_items(X, Y, sym) : npairs, c, chain_ok);
+                if (rc != SK_OK || c.fits) {
+                    if (rc == SK_OK) *bytes = c.total;
+                    return rc;
+                }
+            }
+            BwdPlan b;
+            rc = plan_backward(X, Y, d, dtype, opt, gram ? (sym ? kGramUpper : kGramFull) : kPairsList,
+                               gram ? gram_items(X, Y, sym) : npairs, b);
+            if (rc == SK_OK) *bytes = b.total;
+            return rc;
+        }
+        case SK_OP_BACKWARD_TAPE: {
+            const bool gram = npairs < 0;
+            const bool sym = gram && (opt->flags & SK_FLAG_SYMMETRIC);
+            TapeBwdPlan b;
+            rc = plan_backward_tape(X, Y, d, dtype, opt, gram ? (sym ? kGramUpper : kGramFull) : kPairsList,
+                                    gram ? gram_items(X, Y, sym) : npairs, b, chain_ok);
+            if (rc == SK_OK) *bytes = b.total;
+            return rc;
+        }
+        case SK_OP_MMD2: {
+            // sized by the same planning as sigkernel_mmd2 (X = A, Y = B); npairs = 1 asks for
+            // the gradient's workspace, 0 for the value alone
+            MmdPlan m;
+            rc = plan_mmd2(X, Y, d, dtype, opt, npairs != 0, m, chain_ok);
+            if (rc == SK_OK) *bytes = m.total;
+            return rc;
+        }
+        case SK_OP_MMD2_TEST: {
+            MmdTestPlan t;
+            rc = plan_mmd2_test(X, Y, d, dtype, opt, npairs, t, chain_ok);
+            if (rc == SK_OK) *bytes = t.total;
+            return rc;
+        }
+        default:
+            return fail(SK_ERR_UNSUPPORTED, "workspace for op %d", op);
+    }
+    if (rc == SK_OK) {
+        *bytes = p.total;
+        // sigkernel_forward_tape takes the same workspace and may plan another route
+        const int mode = op == SK_OP_PAIRS ? kPairsList : (opt->flags & SK_FLAG_SYMMETRIC) ? kGramUpper : kGramFull;
+        Plan pt;
+        if (plan_forward(X, Y, d, dtype, opt, mode, p.npairs, pt, false, true, chain) == SK_OK) *bytes = std::max(*bytes, pt.total);
+        t_last_error.clear();
+    }
+    return rc;
 }
 
 }  // namespace
@@ -2029,7 +2151,7 @@ int sigkernel_autotune(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t 
     Cand all[7] = {{1, -1, 1}, {2, -1, 1}, {4, -1, 1}, {1, -1, -1}, {2, -1, -1}, {4, -1, -1}, {0, 1, -1}};
     Cand cands[7];
     int ncand = 0;
-    size_t ws_bytes = 0;
+    size_t ws_bytes = 0, ws_one = 0;  // of all candidates, and of those with one warp per pair (the first ones)
     int rc;
     auto cand_options = [&](const Cand& c) {
         sk_options co = *opt;
@@ -2046,12 +2168,20 @@ int sigkernel_autotune(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t 
         if (all[c].pipe < 0 && all[c].mt > 0 && !p.mtile) continue;  // tiled M not applicable
         cands[ncand++] = all[c];
         ws_bytes = std::max(ws_bytes, p.total);
+        if (all[c].pipe < 0) ws_one = ws_bytes;
     }
     if (n == 0) return fail(SK_ERR_INVALID_ARG, "nothing to tune: no pairs");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     void* ws = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    SK_CUDA(cudaMallocAsync(&ws, ws_bytes, st));
+    OwnedWorkspace owned;
+    rc = owned.take(&ws, ws_bytes, st);
+    if (rc == SK_ERR_WORKSPACE && ncand > 1 && cands[ncand - 1].pipe > 0) {  // no room for the pipeline: without it
+        --ncand;
+        rc = owned.take(&ws, ws_one, st);
+        ws_bytes = ws_one;
+    }
+    if (rc != SK_OK) return rc;
     float best_t = -1.f;
     int best_c = 0;
     rc = SK_OK;
@@ -2080,8 +2210,8 @@ int sigkernel_autotune(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t 
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
-    cudaFreeAsync(ws, st);
     if (rc != SK_OK) return rc;
+    SK_CUDA(owned.release());
     int dev = 0;
     SK_CUDA(cudaGetDevice(&dev));
     const int vw = opt->compute == SK_COMPUTE_F32 ? 4 : 2;
@@ -2117,75 +2247,12 @@ float sigkernel_last_kernel_ms(void) {
 
 int sigkernel_workspace_size(int32_t op, const sk_paths* X, const sk_paths* Y, int32_t d, int64_t npairs,
                              const sk_options* opt, size_t* bytes) {
-    t_last_error.clear();
-    if (!bytes) return fail(SK_ERR_INVALID_ARG, "bytes is NULL");
-    *bytes = 0;
-    if (!opt || !X || !Y) return fail(SK_ERR_INVALID_ARG, "NULL argument");
-    Plan p;
-    int rc;
-    const int dtype = SK_F64;  // sizes do not depend on the input element type
-    switch (op) {
-        case SK_OP_PAIRS:
-            rc = plan_forward(X, Y, d, dtype, opt, kPairsList, npairs, p, true);
-            break;
-        case SK_OP_GRAM: {
-            bool sym = (opt->flags & SK_FLAG_SYMMETRIC) != 0;
-            rc = plan_forward(X, Y, d, dtype, opt, sym ? kGramUpper : kGramFull, gram_items(X, Y, sym), p, true);
-            break;
-        }
-        case SK_OP_BACKWARD: {
-            const bool gram = npairs < 0;
-            const bool sym = gram && (opt->flags & SK_FLAG_SYMMETRIC);
-            if (uses_tape_chunks(opt)) {
-                ChunkBwdPlan c;
-                rc = plan_backward_chunked(X, Y, d, dtype, opt, gram ? (sym ? kGramUpper : kGramFull) : kPairsList,
-                                           gram ? gram_items(X, Y, sym) : npairs, c);
-                if (rc != SK_OK || c.fits) {
-                    if (rc == SK_OK) *bytes = c.total;
-                    return rc;
-                }
-            }
-            BwdPlan b;
-            rc = plan_backward(X, Y, d, dtype, opt, gram ? (sym ? kGramUpper : kGramFull) : kPairsList,
-                               gram ? gram_items(X, Y, sym) : npairs, b);
-            if (rc == SK_OK) *bytes = b.total;
-            return rc;
-        }
-        case SK_OP_BACKWARD_TAPE: {
-            const bool gram = npairs < 0;
-            const bool sym = gram && (opt->flags & SK_FLAG_SYMMETRIC);
-            TapeBwdPlan b;
-            rc = plan_backward_tape(X, Y, d, dtype, opt, gram ? (sym ? kGramUpper : kGramFull) : kPairsList,
-                                    gram ? gram_items(X, Y, sym) : npairs, b);
-            if (rc == SK_OK) *bytes = b.total;
-            return rc;
-        }
-        case SK_OP_MMD2: {
-            // sized by the same planning as sigkernel_mmd2 (X = A, Y = B); npairs = 1 asks for
-            // the gradient's workspace, 0 for the value alone
-            MmdPlan m;
-            rc = plan_mmd2(X, Y, d, dtype, opt, npairs != 0, m);
-            if (rc == SK_OK) *bytes = m.total;
-            return rc;
-        }
-        case SK_OP_MMD2_TEST: {
-            MmdTestPlan t;
-            rc = plan_mmd2_test(X, Y, d, dtype, opt, npairs, t);
-            if (rc == SK_OK) *bytes = t.total;
-            return rc;
-        }
-        default:
-            return fail(SK_ERR_UNSUPPORTED, "workspace for op %d", op);
-    }
-    if (rc == SK_OK) {
-        *bytes = p.total;
-        // sigkernel_forward_tape takes the same workspace and may plan another route
-        const int mode = op == SK_OP_PAIRS ? kPairsList : (opt->flags & SK_FLAG_SYMMETRIC) ? kGramUpper : kGramFull;
-        Plan pt;
-        if (plan_forward(X, Y, d, dtype, opt, mode, p.npairs, pt, false, true) == SK_OK) *bytes = std::max(*bytes, pt.total);
-        t_last_error.clear();
-    }
-    return rc;
+    return workspace(op, X, Y, d, npairs, opt, true, bytes);
+}
+
+int sigkernel_workspace_least(int32_t op, const sk_paths* X, const sk_paths* Y, int32_t d, int64_t npairs,
+                              const sk_options* opt, size_t* bytes) {
+    return workspace(op, X, Y, d, npairs, opt, false, bytes);
 }
 
 int sigkernel_pairs(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, const int64_t* pair_a,

@@ -74,6 +74,8 @@ def load_library():
         lib.sigkernel_last_error.restype = ctypes.c_char_p
         lib.sigkernel_workspace_size.restype = ctypes.c_int
         lib.sigkernel_workspace_size.argtypes = [I32, PP, PP, I32, I64, PO, ctypes.POINTER(SZ)]
+        lib.sigkernel_workspace_least.restype = ctypes.c_int
+        lib.sigkernel_workspace_least.argtypes = lib.sigkernel_workspace_size.argtypes
         lib.sigkernel_pairs.restype = ctypes.c_int
         lib.sigkernel_pairs.argtypes = [PP, PP, I32, I32, P, P, I64, PO, P, P, SZ, P]
         lib.sigkernel_gram.restype = ctypes.c_int
@@ -227,10 +229,18 @@ def _dtype_code(X: Paths, Y: Paths) -> int:
 
 
 def _workspace(op, cX, cY, d, npairs, opt) -> torch.Tensor:
+    """The workspace the call is planned with or, when the device has no room for it, the least one."""
     lib = load_library()
     n = ctypes.c_size_t(0)
-    _check(lib.sigkernel_workspace_size(op, ctypes.byref(cX), ctypes.byref(cY), d, npairs, ctypes.byref(opt),
-                                        ctypes.byref(n)))
+    args = (op, ctypes.byref(cX), ctypes.byref(cY), d, npairs, ctypes.byref(opt), ctypes.byref(n))
+    _check(lib.sigkernel_workspace_size(*args))
+    size = int(n.value)
+    try:
+        return torch.empty(size, dtype=torch.uint8, device="cuda")
+    except torch.cuda.OutOfMemoryError:
+        _check(lib.sigkernel_workspace_least(*args))
+        if int(n.value) >= size:
+            raise
     return torch.empty(int(n.value), dtype=torch.uint8, device="cuda")
 
 
