@@ -182,7 +182,7 @@ struct ChainBuild {
     int nb;                      // buckets of remaining steps per group
     int groups;                  // 1: every item's buffers fit together
     int64_t half;                // units of a group's half of the buffers (groups > 1)
-    unsigned long long* used;    // units taken (groups == 1)
+    unsigned long long* used;    // units taken: in all (groups == 1), or at most in each half
     unsigned int* total;         // tickets
     unsigned int* gsize;         // [groups] tickets
     unsigned int* hist;          // [groups * nb], then the buckets' cursors
@@ -223,7 +223,7 @@ __global__ void chain_base_kernel(Launch L, ChainBuild B) {
 __global__ void chain_group_kernel(Launch L, ChainBuild B) {
     __shared__ int64_t need[1024], at[1024];
     __shared__ int grp[1024];
-    int64_t run = 0;  // thread 0 only
+    int64_t run = 0, most[2] = {0, 0};  // thread 0 only
     int g = 0;
     for (int64_t k0 = 0; k0 < L.npairs; k0 += 1024) {
         const int64_t k = k0 + threadIdx.x;
@@ -241,6 +241,7 @@ __global__ void chain_group_kernel(Launch L, ChainBuild B) {
                 at[q] = run + (g & 1) * B.half;
                 grp[q] = g;
                 run += need[q];
+                if (run > most[g & 1]) most[g & 1] = run;
             }
         __syncthreads();
         if (item >= 0) {
@@ -249,6 +250,8 @@ __global__ void chain_group_kernel(Launch L, ChainBuild B) {
         }
         __syncthreads();
     }
+    if (threadIdx.x == 0)
+        for (int h = 0; h < 2; ++h) B.used[h] = static_cast<unsigned long long>(most[h]);
 }
 
 // One warp per item: lanes take its strips.
@@ -309,12 +312,15 @@ __global__ void chain_scatter_kernel(Launch L, ChainBuild B) {
     }
 }
 
-// Clears the units in use (every unit with more than one group).
-__global__ void chain_clear_kernel(uint4* hand, const unsigned long long* used, int64_t all) {
-    const int64_t n = used ? static_cast<int64_t>(*used) : all;
-    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x)
-        hand[i] = make_uint4(0u, 0u, 0u, 0u);
+// Clears the units in use: used[0] from the start and, with more than one group, used[1] from `half` on.
+// (All 8 GiB of the largest buffers take 1.3 ms.)
+__global__ void chain_clear_kernel(uint4* hand, const unsigned long long* used, int64_t half, int halves) {
+    for (int h = 0; h < halves; ++h) {
+        const int64_t n = static_cast<int64_t>(used[h]);
+        for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
+             i += static_cast<int64_t>(gridDim.x) * blockDim.x)
+            hand[h * half + i] = make_uint4(0u, 0u, 0u, 0u);
+    }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -407,9 +413,9 @@ bool plan_chain(ChainPlan& c, size_t& off, int64_t npairs, int64_t strips, int64
     c.groups = static_cast<int>(groups);
     c.all = groups > 1 ? budget / 2 * 2 : bound;
     c.cols = static_cast<int>(cols);
-    // cleared before each launch: used, total, finished, gsize and gdone, strips done per item, histogram
+    // cleared before each launch: used (two), total, finished, gsize and gdone, strips done per item, histogram
     c.off_counts = off;
-    c.counts_bytes = align256(16 + (2 * static_cast<size_t>(groups) + static_cast<size_t>(npairs) + static_cast<size_t>(nb * groups)) * 4);
+    c.counts_bytes = align256(24 + (2 * static_cast<size_t>(groups) + static_cast<size_t>(npairs) + static_cast<size_t>(nb * groups)) * 4);
     off += c.counts_bytes;
     c.off_base = off;
     off += align256(static_cast<size_t>(npairs) * 8);
@@ -876,8 +882,8 @@ int launch_chain_tickets(const ChainPlan& c, Launch& L, bool sorted, char* base,
     B.groups = c.groups;
     B.half = c.all / 2;
     B.used = reinterpret_cast<unsigned long long*>(counts);
-    B.total = reinterpret_cast<unsigned int*>(counts + 8);
-    B.gsize = reinterpret_cast<unsigned int*>(counts + 16);
+    B.total = reinterpret_cast<unsigned int*>(counts + 16);
+    B.gsize = reinterpret_cast<unsigned int*>(counts + 24);
     unsigned int* gdone = B.gsize + c.groups;
     int* done = reinterpret_cast<int*>(gdone + c.groups);
     B.hist = reinterpret_cast<unsigned int*>(done + L.npairs);
@@ -893,7 +899,7 @@ int launch_chain_tickets(const ChainPlan& c, Launch& L, bool sorted, char* base,
     L.ch_done = done;
     L.ch_gsize = B.gsize;
     L.ch_gdone = gdone;
-    L.ch_finished = reinterpret_cast<int*>(counts + 12);
+    L.ch_finished = reinterpret_cast<int*>(counts + 20);
     L.ch_cols = c.cols;
     L.order = nullptr;
     SK_CUDA(cudaMemsetAsync(counts, 0, c.counts_bytes, st));
@@ -917,7 +923,8 @@ int launch_chain_tickets(const ChainPlan& c, Launch& L, bool sorted, char* base,
     chain_scan_kernel<<<1, 1024, 0, st>>>(B);
     chain_scatter_kernel<<<wb, 256, 0, st>>>(L, B);
     const int cb = static_cast<int>(std::min<int64_t>((c.all + 255) / 256, 4096));
-    chain_clear_kernel<<<cb, 256, 0, st>>>(reinterpret_cast<uint4*>(base + c.off_hand), c.groups == 1 ? B.used : nullptr, c.all);
+    chain_clear_kernel<<<cb, 256, 0, st>>>(reinterpret_cast<uint4*>(base + c.off_hand), B.used, B.half,
+                                       c.groups == 1 ? 1 : 2);
     SK_CUDA(cudaGetLastError());
     return SK_OK;
 }
