@@ -511,6 +511,17 @@ bool chain_pays(const sk_paths* X, const sk_paths* Y, int64_t points, int lam, i
     return chained < 0.9 * one;
 }
 
+bool is_fd(const sk_options* o) {
+    return o->scheme == SK_FD1 || o->scheme == SK_FD2 || o->scheme == SK_FD_IMPLICIT;
+}
+int fd_order(const sk_options* o) { return o->scheme == SK_FD2 ? 2 : o->scheme == SK_FD_IMPLICIT ? 3 : 1; }
+// fd_narrow for a call's longest paths: the same answer for the forward that records a tape and for its adjoint.
+bool narrow_fd(const sk_paths* X, const sk_paths* Y, const sk_options* o, int T, int dpad, bool tape) {
+    const int64_t points = (o->flags & SK_FLAG_INCREMENTS) ? 0 : 1;
+    return fd_narrow(T, fd_order(o), o->dyadic, std::max<int64_t>(X->max_len - points, 1),
+                     std::max<int64_t>(Y->max_len - points, 1), dpad, tape);
+}
+
 // allow_coop: the caller launches p.kern itself with p.threads (the plain forward); adjoint
 // plans reuse this layout with their own one-warp-per-pair kernels and pass false.  tape: the
 // forward records a tape (one warp per pair; its own kernels for the approximation scheme).
@@ -550,7 +561,7 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     p.mtile = mt_eligible && !(o->flags & SK_FLAG_NO_TILED_M);
     auto kernel_for = [&](bool coop) -> const void* {  // coop: the FD schemes' pipelined blocks
         return poly ? fwd_poly_kernel_ptr(p.T, o->scheme == SK_POLY_INTERP, o->degree, false, p.mtile, tape)
-                    : fwd_fd_kernel_ptr(p.T, o->scheme == SK_FD2 ? 2 : o->scheme == SK_FD_IMPLICIT ? 3 : 1, lam, coop, tape);
+                    : fwd_fd_kernel_ptr(p.T, fd_order(o), lam, coop, tape, narrow_fd(X, Y, o, p.T, p.dpad, tape));
     };
     p.kern = kernel_for(false);
     if (poly) {
@@ -819,12 +830,7 @@ struct TapePlan {
     int64_t nsteps_c;  // FD: steps of the coarse-grid schedule of the dk/dM buffer
 };
 
-bool is_fd(const sk_options* o) {
-    return o->scheme == SK_FD1 || o->scheme == SK_FD2 || o->scheme == SK_FD_IMPLICIT;
-}
-int fd_order(const sk_options* o) { return o->scheme == SK_FD2 ? 2 : o->scheme == SK_FD_IMPLICIT ? 3 : 1; }
-
-int plan_tape(const sk_paths* X, const sk_paths* Y, const sk_options* o, int T, int64_t npairs, TapePlan& t) {
+int plan_tape(const sk_paths* X, const sk_paths* Y, const sk_options* o, int T, int dpad, int64_t npairs, TapePlan& t) {
     const int lam = o->dyadic;
     // grid rows and columns of the longest paths: their increments (one fewer than their points)
     const int64_t pts = (o->flags & SK_FLAG_INCREMENTS) ? 0 : 1;
@@ -833,11 +839,12 @@ int plan_tape(const sk_paths* X, const sk_paths* Y, const sk_options* o, int T, 
     int64_t cols = ly << lam;
     int row;
     if (is_fd(o)) {
-        // FD: each lane sweeps 2^lambda node rows (one coarse row), fd_cols refined columns a step
+        // FD: each lane sweeps 2^lambda node rows (one coarse row), fd_tape_cols refined columns a step
         if (lam > 4) return fail(SK_ERR_UNSUPPORTED, "the FD adjoint supports dyadic orders 0..4");
         rows = lx;
-        cols /= fd_tape_cols(lam);
-        row = fd_tape_row_elems(T, lam);
+        const bool narrow = narrow_fd(X, Y, o, T, dpad, true);
+        cols /= fd_tape_cols(lam, narrow);
+        row = fd_tape_row_elems(T, lam, narrow);
     } else {
         const bool interp = o->scheme == SK_POLY_INTERP;
         row = T ? tape_row<float>(o->degree, interp) : tape_row<double>(o->degree, interp);
@@ -938,7 +945,7 @@ int run_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, 
     if (rc != SK_OK) return rc;
     TapePlan tp{0, 0, 0, 0};
     if (tape) {
-        if ((rc = plan_tape(X, Y, o, p.T, npairs, tp)) != SK_OK) return rc;
+        if ((rc = plan_tape(X, Y, o, p.T, p.dpad, npairs, tp)) != SK_OK) return rc;
         if (tape_bytes < tp.total) return fail(SK_ERR_WORKSPACE, "tape %zu bytes < %zu required", tape_bytes, tp.total);
         if (reinterpret_cast<uintptr_t>(tape) % 256) return fail(SK_ERR_INVALID_ARG, "tape must be 256-byte aligned");
     }
@@ -1299,17 +1306,18 @@ int plan_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t 
     int rc = plan_forward(X, Y, d, dtype, o, mode, npairs, b.f, false, false, 0);
     if (rc != SK_OK) return rc;
     const Plan& p = b.f;
-    if ((rc = plan_tape(X, Y, o, p.T, npairs, b.t)) != SK_OK) return rc;
+    if ((rc = plan_tape(X, Y, o, p.T, p.dpad, npairs, b.t)) != SK_OK) return rc;
     const bool interp = o->scheme == SK_POLY_INTERP;
     const bool fd = is_fd(o);
-    b.kern = fd ? bwd_fd_tape_ptr(p.T, fd_order(o), o->dyadic)
+    const bool narrow = fd && narrow_fd(X, Y, o, p.T, p.dpad, true);
+    b.kern = fd ? bwd_fd_tape_ptr(p.T, fd_order(o), o->dyadic, narrow)
                 : (p.T ? bwd_tape_ptr_f32(o->degree, interp) : bwd_tape_ptr_f64(o->degree, interp));
     if (!b.kern) return fail(SK_ERR_UNSUPPORTED, "no adjoint kernel for order %d", o->degree);
     // contraction: every coordinate of a padded increment row in one pass up to 32 (8, 16 or 32)
     b.cC = p.dpad <= 8 ? 8 : (p.dpad <= 16 ? 16 : 32);
     b.ckern = p.T ? bwd_contract_ptr_f32(b.cC) : bwd_contract_ptr_f64(b.cC);
     const int step_bytes = 32 * (p.T ? tape_row<float>(o->degree, interp) * 4 : tape_row<double>(o->degree, interp) * 8);
-    b.smem_bytes = kFwdWarps * (fd ? bwd_fd_ring_bytes(p.T, o->dyadic) : bwd_tape_warp_bytes(step_bytes));
+    b.smem_bytes = kFwdWarps * (fd ? bwd_fd_ring_bytes(p.T, o->dyadic, narrow) : bwd_tape_warp_bytes(step_bytes));
     const int esize = p.T ? 4 : 8, N = fd ? 0 : o->degree;  // FD hands one value per column down
     b.cols_max = std::max<int64_t>(Y->max_len << o->dyadic, 1);
     b.off_rbuf = 0;
@@ -1449,7 +1457,7 @@ int launch_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int32_
     L.scratch_stride = b.slot_bytes;
     L.tau = 1.0f;
     TapePlan tp;  // the tape as the forward laid it out for these npairs items
-    if ((rc = plan_tape(X, Y, o, p.T, npairs, tp)) != SK_OK) return rc;
+    if ((rc = plan_tape(X, Y, o, p.T, p.dpad, npairs, tp)) != SK_OK) return rc;
     L.tape = const_cast<char*>(static_cast<const char*>(tape)) + tp.ek_bytes;
     L.tape_stride = static_cast<int64_t>(tp.stride);
     L.tape_ek = const_cast<int*>(static_cast<const int*>(tape));
@@ -1683,7 +1691,7 @@ int plan_mmd2_blocks(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t d
         Plan p1;
         if ((rc = plan_forward(xs[k], ys[k], d, dtype, ok, modes[k], 1, p1)) != SK_OK) return rc;
         TapePlan t1;
-        if ((rc = plan_tape(xs[k], ys[k], ok, p1.T, 1, t1)) != SK_OK) return rc;
+        if ((rc = plan_tape(xs[k], ys[k], ok, p1.T, p1.dpad, 1, t1)) != SK_OK) return rc;
         TapeBwdPlan whole;
         if ((rc = plan_backward_tape(xs[k], ys[k], d, dtype, ok, modes[k], m.items[k], whole)) != SK_OK) return rc;
         const int64_t resident = whole.resident;
@@ -1707,7 +1715,7 @@ int plan_mmd2_blocks(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t d
             return rc;
         if ((rc = plan_backward_tape(xs[k], ys[k], d, dtype, ok, modes[k], m.chunk[k], m.tb[k], chain_ok)) != SK_OK) return rc;
         TapePlan tc;
-        if ((rc = plan_tape(xs[k], ys[k], ok, p1.T, m.chunk[k], tc)) != SK_OK) return rc;
+        if ((rc = plan_tape(xs[k], ys[k], ok, p1.T, p1.dpad, m.chunk[k], tc)) != SK_OK) return rc;
         m.tape_bytes = std::max(m.tape_bytes, tc.total);
         if (m.items[k] % m.chunk[k]) {  // the last chunk's forward may be planned another way
             Plan last;
@@ -1861,7 +1869,7 @@ int plan_backward_chunked(const sk_paths* X, const sk_paths* Y, int32_t d, int32
     int rc;
     if ((rc = plan_forward(X, Y, d, dtype, o, mode, 1, p1)) != SK_OK) return rc;
     TapePlan t1;
-    if ((rc = plan_tape(X, Y, o, p1.T, 1, t1)) != SK_OK) return rc;
+    if ((rc = plan_tape(X, Y, o, p1.T, p1.dpad, 1, t1)) != SK_OK) return rc;
     TapeBwdPlan whole;
     if ((rc = plan_backward_tape(X, Y, d, dtype, o, mode, std::max<int64_t>(items, 1), whole)) != SK_OK) return rc;
     const int64_t resident = whole.resident;
@@ -1880,7 +1888,7 @@ int plan_backward_chunked(const sk_paths* X, const sk_paths* Y, int32_t d, int32
     if ((rc = plan_forward(X, Y, d, dtype, o, mode, chunk, c.f, false, true, chain_ok ? kChainAny : 0)) != SK_OK) return rc;
     if ((rc = plan_backward_tape(X, Y, d, dtype, o, mode, chunk, c.tb, chain_ok)) != SK_OK) return rc;
     TapePlan tc;
-    if ((rc = plan_tape(X, Y, o, p1.T, chunk, tc)) != SK_OK) return rc;
+    if ((rc = plan_tape(X, Y, o, p1.T, p1.dpad, chunk, tc)) != SK_OK) return rc;
     c.tape_bytes = tc.total;
     const int64_t nout = mode == kPairsList ? chunk : X->count * Y->count;
     c.out_bytes = align256(static_cast<size_t>(std::max<int64_t>(nout, 1)) * sizeof(double));
@@ -2317,7 +2325,7 @@ int sigkernel_tape_size(const sk_paths* X, const sk_paths* Y, int32_t d, int64_t
                           gram ? gram_items(X, Y, sym) : npairs, p);
     if (rc != SK_OK) return rc;
     TapePlan t;
-    if ((rc = plan_tape(X, Y, opt, p.T, p.npairs, t)) != SK_OK) return rc;
+    if ((rc = plan_tape(X, Y, opt, p.T, p.dpad, p.npairs, t)) != SK_OK) return rc;
     *bytes = t.total;
     return SK_OK;
 }

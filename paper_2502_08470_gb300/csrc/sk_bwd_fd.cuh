@@ -40,18 +40,17 @@ __host__ __device__ constexpr int kFdRing() {
     return R <= 1 ? 8 : (R <= 2 ? 6 : 4);
 }
 // Shared-memory bytes of one warp's ring.
-template <typename T, int R>
+template <typename T, int R, int C = fd_cols(R)>
 __host__ __device__ constexpr int fd_ring_warp_bytes() {
-    return kFdRing<R>() * 32 * fd_tape_row<T>(R) * static_cast<int>(sizeof(T));
+    return kFdRing<R>() * 32 * fd_tape_row<T>(R, C) * static_cast<int>(sizeof(T));
 }
 
-template <typename T, int ORDER, int R>
+template <typename T, int ORDER, int R, int C = fd_cols(R)>
 __global__ void __launch_bounds__(kFwdWarps * 32) bwd_fd_tape_kernel(BwdParams B) {
     constexpr bool kRescale = std::is_same<T, float>::value;
     using V = typename Vec<T>::type;
     constexpr int W = Vec<T>::W;
-    constexpr int TR = fd_tape_row<T>(R);
-    constexpr int C = fd_cols(R);
+    constexpr int TR = fd_tape_row<T>(R, C);
     const Launch& L = B.L;
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
@@ -62,7 +61,7 @@ __global__ void __launch_bounds__(kFwdWarps * 32) bwd_fd_tape_kernel(BwdParams B
     constexpr int D = kFdRing<R>();
     constexpr int kStepBytes = 32 * TR * static_cast<int>(sizeof(T));
     extern __shared__ __align__(16) unsigned char fd_smem[];
-    unsigned char* ring = fd_smem + wib * fd_ring_warp_bytes<T, R>();  // [D][vector][lane]
+    unsigned char* ring = fd_smem + wib * fd_ring_warp_bytes<T, R, C>();  // [D][vector][lane]
 
     for (;;) {
         const int64_t item = next_item(L);

@@ -46,7 +46,8 @@ namespace sk {
 
 // Refined columns a lane takes per warp step: the coarse cell's own for 2 or 4 of them, else as many
 // as keep the tile's 16 to 32 sub-cells in registers.  A divisor of 2^lambda for R = min(2^lambda, 16),
-// so that the tile lies in one coarse cell.
+// so that the tile lies in one coarse cell.  FP64 calls on short paths take one column a step instead
+// (fd_narrow).
 __host__ __device__ constexpr int fd_cols(int R) { return R <= 4 ? R : (R == 8 ? 4 : 2); }
 
 // |m| up to which a tile is swept without looking at the magnitudes between its columns: the update
@@ -59,8 +60,8 @@ constexpr float kFdTileM = 1.0f;
 // it the adjoint rebuilds the lane's R x C sub-cells (fd_tape_row elements per lane and step, laid
 // out [vector][lane] like the polynomial tapes).
 template <typename T>
-__host__ __device__ constexpr int fd_tape_row(int R) {
-    return ((R + fd_cols(R) + 3) * static_cast<int>(sizeof(T)) + 15) / 16 * 16 / static_cast<int>(sizeof(T));
+__host__ __device__ constexpr int fd_tape_row(int R, int C) {
+    return ((R + C + 3) * static_cast<int>(sizeof(T)) + 15) / 16 * 16 / static_cast<int>(sizeof(T));
 }
 
 template <typename T>
@@ -75,7 +76,7 @@ __device__ __forceinline__ T fd_pow2(int e) {
 // warp's own when CW = 1).  In a block the hand-off is ordered by the progress words prog[]; a buffer
 // entry of strip g is overwritten by strip g + CW only after strip g + 1 has consumed it, because
 // strip g + CW depends on strip g + 1 through the strips in between.
-template <typename T, int ORDER, int R, int CW, bool TAPE = false>
+template <typename T, int ORDER, int R, int CW, bool TAPE = false, int C = fd_cols(R)>
 __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const PairDesc& P, int w, char* own_buf,
                                          const char* prev_buf, int* prog, int64_t buf_cols) {
     constexpr bool kRescale = std::is_same<T, float>::value;
@@ -89,7 +90,6 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
     const T* __restrict__ incX = static_cast<const T*>(L.X.inc);
     const T* __restrict__ incY = static_cast<const T*>(L.Y.inc);
 
-    constexpr int C = fd_cols(R);
     const int lam = L.lam;
     const int nI = static_cast<int>(P.lx << lam);       // refined node rows 0..nI
     const int nJ = static_cast<int>(P.ly << lam) / C;   // tiles of C refined columns per row group
@@ -170,7 +170,7 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
             if constexpr (TAPE) {  // the tile's inputs for the adjoint (fd_tape_row)
                 using V = typename Vec<T>::type;
                 constexpr int W = Vec<T>::W;
-                constexpr int TR = fd_tape_row<T>(R);
+                constexpr int TR = fd_tape_row<T>(R, C);
                 V* dst = reinterpret_cast<V*>(static_cast<char*>(L.tape) + item * L.tape_stride +
                                               static_cast<int64_t>(step) * (32 * TR * static_cast<int>(sizeof(T))));
 #pragma unroll
@@ -271,7 +271,7 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
 // unconstrained build took (2 blocks per SM).  The pipelined blocks keep their budget: capped at
 // two blocks per SM they ran slower (64 oscillatory pairs at lambda = 4: 30.1 against 22.1 ms).
 // TAPE (CW = 1): also record the forward tape of the FD adjoint (fd_tape_row, L.tape must be set).
-template <typename T, int ORDER, int R, int CW, bool TAPE = false>
+template <typename T, int ORDER, int R, int CW, bool TAPE = false, int C = fd_cols(R)>
 __global__ void __launch_bounds__((CW > 1 ? CW : kFwdWarps) * 32, (CW > 1 ? 1 : (TAPE ? 4 : 8)))
     fwd_fd_kernel(Launch L, int64_t buf_cols) {
     const int wib = threadIdx.x >> 5;
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__((CW > 1 ? CW : kFwdWarps) * 32, (CW > 1 ? 1 : 
         if (item < 0) break;
         const PairDesc P = decode_pair(L, item);
         if (trivial_pair(L, item, P)) continue;
-        sweep_fd<T, ORDER, R, 1, TAPE>(L, item, P, 0, own, own, nullptr, buf_cols);
+        sweep_fd<T, ORDER, R, 1, TAPE, C>(L, item, P, 0, own, own, nullptr, buf_cols);
     }
 }
 
