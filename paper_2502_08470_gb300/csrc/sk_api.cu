@@ -499,14 +499,30 @@ int check_options(const sk_options* o, int32_t d, int32_t dtype) {
 // below it) or the whole batch, with a tenth more instructions a step for the hand-off.  Half the
 // resident warps reach the full FP32 rate, a quarter the FP64 rate.  The batch's total is taken from
 // the mean path lengths, which is all that the host knows.
+// FP64 pairs of one length are counted more exactly, since a block's four warps take all of an SM's FP64
+// rate: one warp per pair takes as long as the SM with the most blocks in each wave (640 pairs of 1025
+// points, order 6: two on some of 152 SMs, 335 ms, where the chain takes 186; the mean over the SMs said
+// 1.05 and left them there), an eighth longer where that is one block, which leaves gaps (order 3: 0.15,
+// order 6: 0.08).  A chain, which spreads evenly, takes the whole batch, a tenth longer with a tape, its
+// fill (576 pairs of 257 points, order 3: 4.36 against 3.70 ms) and its planning kernels, about 20 steps.
+// In FP32 waves blur, and their remainder costs little.
 bool chain_pays(const sk_paths* X, const sk_paths* Y, int64_t points, int lam, int64_t npairs, int64_t strips,
-                int64_t cols, int64_t resident, int T) {
+                int64_t cols, int64_t sms, int64_t per_sm, int T, bool tape) {
     if (X->count <= 0 || Y->count <= 0) return false;
+    const int64_t pair = strips * std::max<int64_t>(cols, 32);
+    if (!T && !uneven_lengths(X) && !uneven_lengths(Y)) {
+        const int64_t blocks = (npairs + kFwdWarps - 1) / kFwdWarps;
+        const int64_t most = blocks / (sms * per_sm) * per_sm + (blocks % (sms * per_sm) + sms - 1) / sms;
+        const double one = static_cast<double>(pair) * (most > 1 ? static_cast<double>(most) : 1.12);
+        const double full = static_cast<double>(npairs) * static_cast<double>(pair) / static_cast<double>(sms * kFwdWarps);
+        const double chained = std::max(static_cast<double>(cols), (tape ? 1.1 : 1.0) * full) + static_cast<double>(kChainLag * strips) + 20.0;
+        return chained < 0.94 * one;
+    }
     const double rx = std::max(1.0, static_cast<double>(X->rows_total) / X->count - points) * (1 << lam);
     const double ry = std::max(1.0, static_cast<double>(Y->rows_total) / Y->count - points) * (1 << lam);
     const double total = static_cast<double>(npairs) * std::ceil(rx / 32.0) * std::max(ry, 32.0);
-    const double full = total / (static_cast<double>(resident) / (T ? 2 : 4));
-    const double one = std::max(static_cast<double>(strips) * std::max<int64_t>(cols, 32), full);
+    const double full = total / (static_cast<double>(sms * per_sm * kFwdWarps) / (T ? 2 : 4));
+    const double one = std::max(static_cast<double>(pair), full);
     const double chained = std::max(static_cast<double>(cols + kChainLag * strips), 1.1 * full);
     return chained < 0.9 * one;
 }
@@ -644,7 +660,7 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     const int64_t strips = (max_rows + 31) / 32;
     if (poly && (allow_coop || tape) && pipe_req >= 0 && strips >= 2 && npairs > 0) {
         want_chain = pipe_req > 0 || chain_pays(X, Y, points, lam, npairs, strips, max_cols,
-                                                static_cast<int64_t>(sms) * per_sm * kFwdWarps, p.T);
+                                                sms, per_sm, p.T, tape);
     }
     // FP64 pairs of one strip, no more of them than SMs: four warps share a pair's cells, since one warp
     // has only a quarter of its SM's FP64 units (sk_fwd_split.cuh).  With two pairs per SM the units
@@ -1383,7 +1399,7 @@ int plan_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t 
     const int units = p.T ? chain_units<float>(N) : chain_units<double>(N);
     if (chain_kern && strips >= 2 && npairs > 0 && chain_ok && !(o->flags & SK_FLAG_NO_STRIP_PIPELINE) &&
         ((o->flags & SK_FLAG_STRIP_PIPELINE) || chain_pays(X, Y, points, o->dyadic, npairs, strips, max_cols,
-                                                           static_cast<int64_t>(sms) * per_sm * kFwdWarps, p.T))) {
+                                                           sms, per_sm, p.T, true))) {
         int cper = 0;
         SK_CUDA(cudaFuncSetAttribute(chain_kern, cudaFuncAttributeMaxDynamicSharedMemorySize, b.smem_bytes));
         SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cper, chain_kern, p.threads, b.smem_bytes));
