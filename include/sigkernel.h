@@ -288,8 +288,10 @@ int sigkernel_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int
  * sigkernel_autotune -- choose the launch shape of a forward call (sigkernel_pairs when pair_a is
  * non-NULL, else sigkernel_gram; same arguments) by timing the candidates on these inputs:
  * one warp per pair in blocks of 1, 2 or 4 warps (each with and without the tiled M where it
- * applies), and the strip pipeline (SK_FLAG_STRIP_PIPELINE: several warps share each pair of two or
- * more strips) when some pair spans two strips.  Each candidate runs
+ * applies), four warps sharing each pair where the library does so by itself (FP64, pairs of one strip,
+ * no more of them than SMs: warps_per_block 0 and no strip-pipeline flag), and the strip pipeline
+ * (SK_FLAG_STRIP_PIPELINE: several warps share each pair of two or more strips) when some pair spans
+ * two strips.  Each candidate runs
  * once to warm up, then `trials` (1..1000) timed times on `stream`; `out` is overwritten with the
  * results.  The call allocates its own workspace (stream-ordered) and returns after the runs have
  * finished on the device.

@@ -56,9 +56,10 @@ struct TuneKey {
     }
 };
 struct TuneChoice {
-    int wpb;   // warps per block of the one-warp-per-pair kernel
-    int pipe;  // 1: strip pipeline, -1: none
-    int mt;    // 1: tiled M where eligible, -1: per-cell M
+    int wpb;     // warps per block of the one-warp-per-pair kernel
+    int pipe;    // 1: strip pipeline, -1: none
+    int mt;      // 1: tiled M where eligible, -1: per-cell M
+    bool split;  // FP64 pairs of one strip: four warps per pair
 };
 std::mutex g_tune_mu;
 std::map<TuneKey, TuneChoice> g_tune;
@@ -588,6 +589,7 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     // Launch shape.  Explicit requests (warps_per_block, the strip-pipeline flags) win; otherwise a
     // shape that sigkernel_autotune measured for this shape of call; otherwise the defaults.
     int wpb_req = 0, pipe_req = 0;  // pipe_req: 1 strip pipeline, -1 none, 0 the default rule
+    bool split_ok = o->warps_per_block == 0 && !(o->flags & (SK_FLAG_STRIP_PIPELINE | SK_FLAG_NO_STRIP_PIPELINE));
     if (allow_coop) wpb_req = o->warps_per_block;
     if (allow_coop || tape) {
         if (o->flags & SK_FLAG_STRIP_PIPELINE) pipe_req = 1;
@@ -602,6 +604,7 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
         if (it != g_tune.end()) {
             wpb_req = it->second.wpb;
             pipe_req = it->second.pipe;
+            split_ok = it->second.split;
             if (it->second.mt < 0 && p.mtile) {
                 p.mtile = false;
                 p.kern = kernel_for(false);
@@ -665,8 +668,7 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     // FP64 pairs of one strip, no more of them than SMs: four warps share a pair's cells, since one warp
     // has only a quarter of its SM's FP64 units (sk_fwd_split.cuh).  With two pairs per SM the units
     // would be shared all the same, and the exchange between the warps would only cost.
-    const bool shape_asked = o->warps_per_block != 0 || (o->flags & (SK_FLAG_STRIP_PIPELINE | SK_FLAG_NO_STRIP_PIPELINE));
-    if (poly && !p.T && allow_coop && !shape_asked && strips == 1 && npairs > 0 && npairs <= sms) {
+    if (poly && !p.T && allow_coop && split_ok && strips == 1 && npairs > 0 && npairs <= sms) {
         const void* sk = fwd_split_ptr_f64(o->scheme == SK_POLY_INTERP, o->degree);
         int sper = 0;
         if (sk && (rc = occupancy(sk, kSplitWarps * 32, &sper)) != SK_OK) return rc;
@@ -2177,24 +2179,33 @@ int sigkernel_autotune(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t 
     const int strip = SK_FLAG_STRIP_PIPELINE | SK_FLAG_NO_STRIP_PIPELINE | SK_FLAG_TIME_KERNEL;
     struct Cand {
         int wpb, pipe, mt;
+        bool split;
     };
-    // one warp per pair with 1, 2, 4 warps per block, with and without tiled M; the pipeline
-    Cand all[7] = {{1, -1, 1}, {2, -1, 1}, {4, -1, 1}, {1, -1, -1}, {2, -1, -1}, {4, -1, -1}, {0, 1, -1}};
-    Cand cands[7];
+    // one warp per pair with 1, 2, 4 warps per block, with and without tiled M; four warps per pair, which
+    // is the library's own choice where it applies (no shape asked for); the pipeline
+    Cand all[8] = {{1, -1, 1, false},  {2, -1, 1, false},  {4, -1, 1, false}, {1, -1, -1, false},
+                   {2, -1, -1, false}, {4, -1, -1, false}, {0, -1, -1, true}, {0, 1, -1, false}};
+    Cand cands[8];
     int ncand = 0;
     size_t ws_bytes = 0, ws_one = 0;  // of all candidates, and of those with one warp per pair (the first ones)
     int rc;
     auto cand_options = [&](const Cand& c) {
         sk_options co = *opt;
+        if (c.split) {  // (with the tiled-M flag, which FP64 ignores, no remembered shape is looked up)
+            co.flags = (opt->flags & ~strip) | SK_FLAG_NO_TILED_M;
+            co.warps_per_block = 0;
+            return co;
+        }
         co.flags = (opt->flags & ~(strip | SK_FLAG_NO_TILED_M)) |
                    (c.pipe > 0 ? SK_FLAG_STRIP_PIPELINE : SK_FLAG_NO_STRIP_PIPELINE) | (c.mt < 0 ? SK_FLAG_NO_TILED_M : 0);
         co.warps_per_block = c.wpb;
         return co;
     };
-    for (int c = 0; c < 7; ++c) {
+    for (int c = 0; c < 8; ++c) {
         sk_options co = cand_options(all[c]);
         Plan p;
         if ((rc = plan_forward(X, Y, d, dtype, &co, mode, n, p, true)) != SK_OK) return rc;
+        if (all[c].split && !p.split) continue;
         if (all[c].pipe > 0 && !p.coop && !p.chain.on) continue;  // no pair spans two strips
         if (all[c].pipe < 0 && all[c].mt > 0 && !p.mtile) continue;  // tiled M not applicable
         cands[ncand++] = all[c];
@@ -2250,7 +2261,8 @@ int sigkernel_autotune(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t 
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         g_tune[tune_key(dev, X, Y, opt, dpad, mode, n)] =
-            TuneChoice{cands[best_c].wpb ? cands[best_c].wpb : kFwdWarps, cands[best_c].pipe, cands[best_c].mt};
+            TuneChoice{cands[best_c].wpb ? cands[best_c].wpb : kFwdWarps, cands[best_c].pipe, cands[best_c].mt,
+                       cands[best_c].split};
     }
     *best = cand_options(cands[best_c]);
     if (best_ms) *best_ms = best_t;

@@ -315,7 +315,8 @@ def autotune(X, Y=None, pair_a=None, pair_b=None, scheme="approx", degree=6, dya
              trials=3, sort=True):
     """Time the forward launch shapes on these inputs (``sigkernel_autotune``) and remember the
     fastest for later calls of the same shape that leave the shape to the library.  Returns
-    ``(shape, ms)`` with ``shape = {"warps_per_block": w, "strip_pipeline": bool}``."""
+    ``(shape, ms)`` with ``shape = {"warps_per_block": w, "strip_pipeline": bool}`` (w = 0: four warps
+    share each pair, FP64 pairs of one strip)."""
     pairs = pair_a is not None
     sym = not pairs and (Y is None or Y is X)
     X = as_paths(X)
