@@ -101,7 +101,8 @@ enum {
     SK_FLAG_SYMMETRIC = 1,    /* sigkernel_gram: Y is X; only a <= b is computed and mirrored */
     SK_FLAG_INCREMENTS = 2,   /* rows hold increments, not points */
     SK_FLAG_UNBIASED = 4,     /* sigkernel_mmd2: U-statistic (diagonals of K_AA, K_BB left out) */
-    SK_FLAG_NO_SORT = 8,      /* process pairs in the given order (no cell-count ordering) */
+    SK_FLAG_NO_SORT = 8,      /* process pairs in the given order (no cell-count ordering; saves its
+                                 launches where all pairs have the same number of cells) */
     SK_FLAG_TIME_KERNEL = 16, /* record CUDA events around the wavefront kernel(s) of this call on
                                  `stream`; read the duration with sigkernel_last_kernel_ms() */
     SK_FLAG_STRIP_PIPELINE = 32,    /* sweep every pair of 2 or more strips (32 grid rows each) by

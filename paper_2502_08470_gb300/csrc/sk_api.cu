@@ -327,12 +327,15 @@ __global__ void chain_clear_kernel(uint4* hand, const unsigned long long* used, 
 // ------------------------------------------------------------------------------------------
 // Argument checks and workspace planning.
 // ------------------------------------------------------------------------------------------
-// Whether ordering the items by cell count can matter: not when every path is as long as the longest
-// (as many rows as that takes).  The order is a schedule only; results do not depend on it.
+// Whether some path is shorter than the longest, as far as the row count says (a set may have rows that no
+// path takes).
 bool uneven_lengths(const sk_paths* S) { return S->rows_total < S->count * S->max_len; }
-bool sort_items(const sk_paths* X, const sk_paths* Y, const sk_options* o, int64_t items) {
-    return !(o->flags & SK_FLAG_NO_SORT) && items > 1 && (uneven_lengths(X) || uneven_lengths(Y));
-}
+// Whether to order the items by cell count.  Only the caller can know that all paths are equally long
+// (the offsets are on the device) and say so with SK_FLAG_NO_SORT, which saves three launches: with the
+// rows per path as the sign, ragged sets in a buffer with room left went unsorted, and the FD pipeline,
+// whose blocks leave off sharing pairs at the first short one, swept the long ones after it by single
+// warps.
+bool sort_items(const sk_options* o, int64_t items) { return !(o->flags & SK_FLAG_NO_SORT) && items > 1; }
 
 // Strip chain of a launch (sk_chain.cuh).
 struct ChainPlan {
@@ -1062,7 +1065,7 @@ int run_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, 
         SK_CUDA(cudaMemsetAsync(base + p.off_queue, 0, 256 + align256(2 * 65 * sizeof(unsigned int)), st));
         if (p.chain.on) {
             if ((rc = launch_chain_tickets(p.chain, C, !(o->flags & SK_FLAG_NO_SORT), base, p.off_hist, p.off_order, st)) != SK_OK) return rc;
-        } else if (sort_items(X, Y, o, n)) {
+        } else if (sort_items(o, n)) {
             unsigned int* hist = reinterpret_cast<unsigned int*>(base + p.off_hist);
             int32_t* order = reinterpret_cast<int32_t*>(base + p.off_order);
             int sb = static_cast<int>((n + 255) / 256);
@@ -1227,7 +1230,7 @@ int launch_backward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dty
     B.off_rexp = b.off_rexp;
     B.off_ybar = b.off_ybar;
     SK_CUDA(cudaMemsetAsync(base + p.off_queue, 0, 256 + align256(2 * 65 * sizeof(unsigned int)), st));
-    if (sort_items(X, Y, o, npairs)) {
+    if (sort_items(o, npairs)) {
         unsigned int* hist = reinterpret_cast<unsigned int*>(base + p.off_hist);
         int32_t* order = reinterpret_cast<int32_t*>(base + p.off_order);
         int sb = static_cast<int>(std::min<int64_t>((npairs + 255) / 256, 4096));
@@ -1502,7 +1505,7 @@ int launch_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int32_
     SK_CUDA(cudaMemsetAsync(base + p.off_queue, 0, 256 + align256(2 * 65 * sizeof(unsigned int)), st));
     if (b.chain.on) {
         if ((rc = launch_chain_tickets(b.chain, L, !(o->flags & SK_FLAG_NO_SORT), base, p.off_hist, p.off_order, st)) != SK_OK) return rc;
-    } else if (sort_items(X, Y, o, npairs)) {
+    } else if (sort_items(o, npairs)) {
         unsigned int* hist = reinterpret_cast<unsigned int*>(base + p.off_hist);
         int32_t* order = reinterpret_cast<int32_t*>(base + p.off_order);
         int sb = static_cast<int>(std::min<int64_t>((npairs + 255) / 256, 4096));

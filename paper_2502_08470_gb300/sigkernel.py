@@ -115,11 +115,13 @@ def _check(rc: int):
 @dataclass
 class Paths:
     """A ragged batch of paths: ``rows`` [R, d] (points, or increments with ``increments=True``)
-    on the GPU and int64 ``offsets`` [B + 1] (path a is rows offsets[a]:offsets[a+1])."""
+    on the GPU and int64 ``offsets`` [B + 1] (path a is rows offsets[a]:offsets[a+1]).  ``equal`` says
+    that every path has ``max_len`` rows: calls on such sets leave out ordering the pairs by size."""
     rows: torch.Tensor
     offsets: torch.Tensor
     max_len: int
     increments: bool = False
+    equal: bool = False
 
     @property
     def count(self) -> int:
@@ -138,13 +140,14 @@ class Paths:
         if ts:
             off[1:] = torch.cumsum(torch.tensor(lens, dtype=torch.int64), 0)
         rows = torch.cat([t.to(dtype) for t in ts], 0) if ts else torch.zeros(0, 1, dtype=dtype)
-        return Paths(rows.to(device).contiguous(), off.to(device), max(lens) if lens else 0, increments)
+        return Paths(rows.to(device).contiguous(), off.to(device), max(lens) if lens else 0, increments,
+                     len(set(lens)) <= 1)
 
     @staticmethod
     def from_dense(x: torch.Tensor, increments=False) -> "Paths":
         B, L, d = x.shape
         off = torch.arange(0, (B + 1) * L, L, dtype=torch.int64, device=x.device)
-        return Paths(x.reshape(B * L, d).contiguous(), off, L, increments)
+        return Paths(x.reshape(B * L, d).contiguous(), off, L, increments, True)
 
 
 def as_paths(x) -> Paths:
@@ -244,6 +247,11 @@ def _workspace(op, cX, cY, d, npairs, opt) -> torch.Tensor:
     return torch.empty(int(n.value), dtype=torch.uint8, device="cuda")
 
 
+def _sort_flag(sort: bool, X: Paths, Y: Paths) -> int:
+    """FLAG_NO_SORT when the caller wants the given order, or when all pairs have as many cells."""
+    return 0 if sort and not (X.equal and Y.equal) else FLAG_NO_SORT
+
+
 def _flags(X: Paths, extra=0) -> int:
     return extra | (FLAG_INCREMENTS if X.increments else 0)
 
@@ -259,7 +267,7 @@ def sigkernel_pairs(X, Y, pair_a, pair_b, scheme="approx", degree=6, dyadic=0, c
     pa, pb = _pair_tensors(pair_a, pair_b)
     n = pa.numel()
     opt = _options(scheme, degree, dyadic, compute,
-                   _flags(X, (0 if sort else FLAG_NO_SORT) | _pipe_flags(strip_pipeline)
+                   _flags(X, _sort_flag(sort, X, Y) | _pipe_flags(strip_pipeline)
                           | (FLAG_TIME_KERNEL if time_kernel else 0) | (0 if tiled_m else FLAG_NO_TILED_M)
                           | (0 if tensor_cores else FLAG_NO_TC)))
     cX, cY = _cpaths(X), _cpaths(Y)
@@ -286,7 +294,7 @@ def sigkernel_gram(X, Y=None, scheme="approx", degree=6, dyadic=0, compute="f64"
     sym = Y is None or Y is X
     X = as_paths(X)
     Y = X if sym else as_paths(Y)
-    flags = _flags(X, (FLAG_SYMMETRIC if sym else 0) | (0 if sort else FLAG_NO_SORT)
+    flags = _flags(X, (FLAG_SYMMETRIC if sym else 0) | _sort_flag(sort, X, Y)
                    | (FLAG_TIME_KERNEL if time_kernel else 0) | _pipe_flags(strip_pipeline)
                    | (0 if tiled_m else FLAG_NO_TILED_M) | (0 if tensor_cores else FLAG_NO_TC))
     opt = _options(scheme, degree, dyadic, compute, flags)
@@ -330,7 +338,7 @@ def autotune(X, Y=None, pair_a=None, pair_b=None, scheme="approx", degree=6, dya
         n, pa_ptr, pb_ptr = 0, None, None
         out = torch.empty(X.count, Y.count, dtype=torch.float64, device="cuda")
     opt = _options(scheme, degree, dyadic, compute,
-                   _flags(X, (FLAG_SYMMETRIC if sym else 0) | (0 if sort else FLAG_NO_SORT)))
+                   _flags(X, (FLAG_SYMMETRIC if sym else 0) | _sort_flag(sort, X, Y)))
     best = _Options()
     ms = ctypes.c_float(0)
     _check(load_library().sigkernel_autotune(ctypes.byref(cX), ctypes.byref(cY), X.d, _dtype_code(X, Y), pa_ptr,
@@ -364,7 +372,7 @@ def sigkernel_backward(grad_out, X, Y=None, pair_a=None, pair_b=None, scheme="ap
     gX = torch.zeros(X.rows.shape[0], X.d, dtype=torch.float64, device="cuda")
     same = sym or (X.rows.data_ptr() == Y.rows.data_ptr() and X.offsets.data_ptr() == Y.offsets.data_ptr())
     gY = gX if same else torch.zeros(Y.rows.shape[0], Y.d, dtype=torch.float64, device="cuda")
-    extra = ((0 if sort else FLAG_NO_SORT) | (FLAG_TIME_KERNEL if time_kernel else 0) | (FLAG_CHECKPOINT if checkpoint else 0)
+    extra = (_sort_flag(sort, X, Y) | (FLAG_TIME_KERNEL if time_kernel else 0) | (FLAG_CHECKPOINT if checkpoint else 0)
              | (0 if tensor_cores else FLAG_NO_TC))
     if pair_a is None:
         opt = _options(scheme, degree, dyadic, compute, _flags(X, extra | (FLAG_SYMMETRIC if sym else 0)))
@@ -401,7 +409,7 @@ def sigkernel_forward_tape(X, Y=None, pair_a=None, pair_b=None, scheme="approx",
     Y = X if (Y is None or Y is X) else as_paths(Y)
     cX, cY = _cpaths(X), _cpaths(Y)
     pa_ptr, pb_ptr, n, keep = _pair_args(X, pair_a, pair_b, sym)
-    flags = _flags(X, (FLAG_SYMMETRIC if sym else 0) | (0 if sort else FLAG_NO_SORT)
+    flags = _flags(X, (FLAG_SYMMETRIC if sym else 0) | _sort_flag(sort, X, Y)
                    | (FLAG_TIME_KERNEL if time_kernel else 0) | (0 if tensor_cores else FLAG_NO_TC))
     opt = _options(scheme, degree, dyadic, compute, flags)
     lib = load_library()
@@ -430,7 +438,7 @@ def sigkernel_backward_tape(tape, grad_out, X, Y=None, pair_a=None, pair_b=None,
     Y = X if (Y is None or Y is X) else as_paths(Y)
     cX, cY = _cpaths(X), _cpaths(Y)
     pa_ptr, pb_ptr, n, keep = _pair_args(X, pair_a, pair_b, sym)
-    flags = _flags(X, (FLAG_SYMMETRIC if sym else 0) | (0 if sort else FLAG_NO_SORT)
+    flags = _flags(X, (FLAG_SYMMETRIC if sym else 0) | _sort_flag(sort, X, Y)
                    | (FLAG_TIME_KERNEL if time_kernel else 0) | (0 if tensor_cores else FLAG_NO_TC))
     opt = _options(scheme, degree, dyadic, compute, flags)
     g = _grad_out(grad_out, X.count, Y.count, n)
@@ -446,13 +454,18 @@ def sigkernel_backward_tape(tape, grad_out, X, Y=None, pair_a=None, pair_b=None,
     return gX, gY
 
 
+def _mmd_sort_flag(A: Paths, B: Paths) -> int:
+    """MMD^2 pairs the paths of both sets with one another: FLAG_NO_SORT when all of them are as long."""
+    return FLAG_NO_SORT if A.equal and B.equal and A.max_len == B.max_len else 0
+
+
 def sigkernel_mmd2(A, B, scheme="approx", degree=6, dyadic=0, compute="f64", unbiased=False, grads=False,
                    tensor_cores: bool = True):
     """MMD^2 between path sets A and B; returns (mmd2, [mean K_AA, mean K_BB, mean K_AB]) or, with
     ``grads``, also (dMMD2/dA rows, dMMD2/dB rows) as float64 CUDA tensors."""
     A, B = as_paths(A), as_paths(B)
     cA, cB = _cpaths(A), _cpaths(B)
-    opt = _options(scheme, degree, dyadic, compute, _flags(A, (FLAG_UNBIASED if unbiased else 0)
+    opt = _options(scheme, degree, dyadic, compute, _flags(A, (FLAG_UNBIASED if unbiased else 0) | _mmd_sort_flag(A, B)
                                                            | (0 if tensor_cores else FLAG_NO_TC)))
     ws = _workspace(OP_MMD2, cA, cB, A.d, 1 if grads else 0, opt)
     out = torch.empty(4, dtype=torch.float64, device="cuda")
@@ -493,7 +506,7 @@ def sigkernel_mmd2_test(A, B, permutations=1000, labels=None, seed=0, scheme="ap
     labels = _device_buffer(labels.contiguous(), "labels", torch.uint8, labels.shape[0] * (A.count + B.count))
     nperm = labels.shape[0]
     cA, cB = _cpaths(A), _cpaths(B)
-    opt = _options(scheme, degree, dyadic, compute, _flags(A, FLAG_UNBIASED if unbiased else 0))
+    opt = _options(scheme, degree, dyadic, compute, _flags(A, (FLAG_UNBIASED if unbiased else 0) | _mmd_sort_flag(A, B)))
     ws = _device_buffer(workspace, "workspace") if workspace is not None else \
         _workspace(OP_MMD2_TEST, cA, cB, A.d, nperm, opt)
     if out is None:
@@ -508,7 +521,7 @@ def sigkernel_mmd2_test(A, B, permutations=1000, labels=None, seed=0, scheme="ap
 def mmd2_test_workspace(A, B, nperm, scheme="approx", degree=6, dyadic=0, compute="f64", unbiased=False):
     """Device workspace of ``sigkernel_mmd2_test`` for these sets and relabelling count."""
     A, B = as_paths(A), as_paths(B)
-    opt = _options(scheme, degree, dyadic, compute, _flags(A, FLAG_UNBIASED if unbiased else 0))
+    opt = _options(scheme, degree, dyadic, compute, _flags(A, (FLAG_UNBIASED if unbiased else 0) | _mmd_sort_flag(A, B)))
     return _workspace(OP_MMD2_TEST, _cpaths(A), _cpaths(B), A.d, int(nperm), opt)
 
 
