@@ -440,6 +440,15 @@ constexpr int bwd_min_blocks() {
     return sizeof(T) == 8 ? 1 : (DMAX <= 8 ? 5 : 3);
 }
 
+// <dx_i, dy_j> of the checkpointing adjoint.  FP32 orders 5 and 6 just fit their registers and keep the loop:
+// without it order 6 spills 60 bytes instead of 12 (3000 pairs of 257 points, d = 4, 9.87 against 9.50 ms);
+// the other orders gain 1 to 5% (order 3, 6.35 -> 6.12 ms).
+template <typename T, int N>
+__device__ __forceinline__ T ckpt_dot(const T* __restrict__ x, const T* __restrict__ y, int nvec) {
+    if constexpr (sizeof(T) == 4 && (N == 5 || N == 6)) return row_dot_loop<T>(x, y, nvec);
+    else return row_dot<T>(x, y, nvec);
+}
+
 template <typename T, int N, int K, int DMAX>
 __global__ void __launch_bounds__(kFwdWarps * 32, (bwd_min_blocks<T, N, K, DMAX>()))
     bwd_approx_kernel(BwdParams B) {
@@ -527,8 +536,8 @@ __global__ void __launch_bounds__(kFwdWarps * 32, (bwd_min_blocks<T, N, K, DMAX>
                         ea = 0;
                     }
                     if (kRescale) align_inputs<T, N>(a, ea, b, eb);
-                    const T M = row_dot<T>(xbase + static_cast<int64_t>(row >> lam) * dpad,
-                                           ybase + static_cast<int64_t>(jj >> lam) * dpad, L.nvec) * sub;
+                    const T M = ckpt_dot<T, N>(xbase + static_cast<int64_t>(row >> lam) * dpad,
+                                               ybase + static_cast<int64_t>(jj >> lam) * dpad, L.nvec) * sub;
                     fwd_cell<T, N>(a, b, M, L.tau, bo, ea);
                     if (row == rows - 1 && jj == cols - 1) {
                         double v = 0.5 * (series_at_one<T, N>(a) + series_at_one<T, N>(bo));
@@ -601,7 +610,7 @@ __global__ void __launch_bounds__(kFwdWarps * 32, (bwd_min_blocks<T, N, K, DMAX>
                             ea = 0;
                         }
                         if (kRescale) align_inputs<T, N>(a, ea, b, eb);
-                        const T M = row_dot<T>(xrow, ybase + static_cast<int64_t>(jj >> lam) * dpad, L.nvec) * sub;
+                        const T M = ckpt_dot<T, N>(xrow, ybase + static_cast<int64_t>(jj >> lam) * dpad, L.nvec) * sub;
                         T e[N + 1], ct[N + 1], cr[N + 1], da[N], db[N];
                         build_exp_series<T, N>(M, L.tau, e);
                         cell_series_dm<T, N>(a, b, e, ct, cr, da, db);  // ct, cr: fwd_cell's outputs

@@ -81,10 +81,19 @@ template <> struct Vec<double> {
     }
 };
 
-// <dx_i, dy_j> over `nvec` 16-byte chunks of zero-padded increment rows (read-only path).  One or two
-// chunks, the common widths, go without a loop, whose counters and branches took more instructions than
-// the products: FD2, lambda = 2, 128 x 128 Gram of 129-point paths, d = 8, 2.87 -> 2.55 ms; order 6,
-// 150-path symmetric Gram of 100-point paths, d = 3, 1.29 -> 1.23 ms.
+// <dx_i, dy_j> over `nvec` 16-byte chunks of zero-padded increment rows (read-only path).
+template <typename T>
+__device__ __forceinline__ T row_dot_loop(const T* __restrict__ x, const T* __restrict__ y, int nvec) {
+    using V = typename Vec<T>::type;
+    const V* xv = reinterpret_cast<const V*>(x);
+    const V* yv = reinterpret_cast<const V*>(y);
+    T acc = T(0);
+    for (int c = 0; c < nvec; ++c) acc = Vec<T>::dot(__ldg(xv + c), __ldg(yv + c), acc);
+    return acc;
+}
+// The same without a loop for one or two chunks, the common widths: its counters and branches took more
+// instructions than the products.  FD2, lambda = 2, 128 x 128 Gram of 129-point paths, d = 8, 2.87 ->
+// 2.55 ms; order 6, 150-path symmetric Gram of 100-point paths, d = 3, 1.29 -> 1.23 ms.
 template <typename T>
 __device__ __forceinline__ T row_dot(const T* __restrict__ x, const T* __restrict__ y, int nvec) {
     using V = typename Vec<T>::type;
@@ -95,9 +104,7 @@ __device__ __forceinline__ T row_dot(const T* __restrict__ x, const T* __restric
         const V x0 = __ldg(xv), y0 = __ldg(yv), x1 = __ldg(xv + 1), y1 = __ldg(yv + 1);
         return Vec<T>::dot(x1, y1, Vec<T>::dot(x0, y0, T(0)));
     }
-    T acc = T(0);
-    for (int c = 0; c < nvec; ++c) acc = Vec<T>::dot(__ldg(xv + c), __ldg(yv + c), acc);
-    return acc;
+    return row_dot_loop<T>(x, y, nvec);
 }
 
 // Row i of increments whose rows take row_bytes bytes: one 32 x 32 + 64-bit multiply-add, where i times
