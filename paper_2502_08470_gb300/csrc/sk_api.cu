@@ -387,8 +387,9 @@ constexpr int kPlainSmem = 32 * 1024;
 // wrote before the chunk's sweep); a chunk is a whole number of the sweep's resident warps.
 constexpr size_t kMxBudget = size_t(8) << 30;
 // Bytes of hand-off buffers a strip chain may take, the fewest buffers a pair with more strips may
-// use in turn, and the most buckets its tickets are sorted into.  8 GB holds every buffer of 4096
-// uneven pairs of 64 .. 4096 points (7.7 GB at N = 6 in FP32).
+// use in turn, and the most buckets its tickets are sorted into.  The budget is a thirtieth of the
+// memory; pairs beyond it go in groups, which wait for one another, and a call that finds no room for it
+// takes less (plan_forward_within).
 constexpr size_t kChainBudget = size_t(8) << 30;
 constexpr int64_t kChainMinRing = 64;
 constexpr int64_t kChainMaxBuckets = 1 << 16;
@@ -788,17 +789,23 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
 
 // Blocks of 128 threads over every element of a path set's rows: paths, and as many pieces of a path as
 // give the GPU about 16 such blocks per SM, at four elements a thread or more.
-dim3 path_grid(const sk_paths* S, int width) {
+int path_grid(const sk_paths* S, int width, dim3* grid) {
+    int dev = 0, sms = 0;
+    SK_CUDA(cudaGetDevice(&dev));
+    SK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int64_t x = std::min<int64_t>(S->count, 65535);
-    const int64_t y = std::min<int64_t>((S->max_len * width + 511) / 512, std::max<int64_t>(2432 / x, 1) * 2);
-    return dim3(static_cast<unsigned>(x), static_cast<unsigned>(std::max<int64_t>(y, 1)));
+    const int64_t y = std::min<int64_t>((S->max_len * width + 511) / 512, std::max<int64_t>(16 * sms / x, 1) * 2);
+    *grid = dim3(static_cast<unsigned>(x), static_cast<unsigned>(std::max<int64_t>(y, 1)));
+    return SK_OK;
 }
 
 template <typename T>
 int launch_increments(const sk_paths* S, int32_t d, int32_t dtype, int inc_mode, int dpad, void* out,
                       cudaStream_t st) {
     if (S->count == 0) return SK_OK;
-    const dim3 blocks = path_grid(S, dpad);
+    dim3 blocks;
+    const int rc = path_grid(S, dpad, &blocks);
+    if (rc != SK_OK) return rc;
     T* o = static_cast<T*>(out);
     switch (dtype) {
         case SK_F64:
@@ -1258,7 +1265,10 @@ int launch_backward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dty
 int convert_grad(const sk_paths* S, int32_t d, int dpad, int inc_mode, const double* ginc, double* grad,
                  cudaStream_t st) {
     if (!grad || S->count == 0) return SK_OK;
-    inc_to_row_grad_kernel<<<path_grid(S, d), 128, 0, st>>>(ginc, S->offsets, S->count, S->rows_total, S->max_len, d, dpad,
+    dim3 blocks;
+    const int rc = path_grid(S, d, &blocks);
+    if (rc != SK_OK) return rc;
+    inc_to_row_grad_kernel<<<blocks, 128, 0, st>>>(ginc, S->offsets, S->count, S->rows_total, S->max_len, d, dpad,
                                                    inc_mode, grad);
     SK_CUDA(cudaGetLastError());
     return SK_OK;

@@ -30,7 +30,7 @@
 // everything else a step does: exponents, shuffles, the inner product, index arithmetic and the
 // hand-off (209 issue slots per warp step of 4 sub-cells a lane at lambda = 2).  A step of R x C
 // sub-cells pays for these once and forms the one m they share once.  Measured: FD2, lambda = 2,
-// 128 x 128 Gram of 129-point paths, d = 8, FP32, 6.24 -> 2.87 ms with 4 columns a step, 302 warp
+// 128 x 128 Gram of 129-point paths, d = 8, FP32, 6.24 -> 2.87 ms with 4 columns a step, then 302 warp
 // instructions a step (112 of them the 16 sub-cells) at 0.76 issued a cycle: bound by issue.  Inner
 // products without a loop (2.55 ms) and the row's index, test and increments kept over a strip instead
 // of formed each step (2.35 ms) took more of them out.  FD2, lambda = 1, 48 x 48 pairs, forward with
@@ -51,8 +51,9 @@ namespace sk {
 __host__ __device__ constexpr int fd_cols(int R) { return R <= 4 ? R : (R == 8 ? 4 : 2); }
 
 // |m| up to which a tile is swept without looking at the magnitudes between its columns: the update
-// then multiplies a node by less than 4, the longest chain of updates in a tile has R + C - 1 <= 17
-// of them, and values start within [2^-64, 2^64].  Above it the tile is rescaled after every column.
+// then makes a node less than 4.4 times the largest of the three it comes from (4.33 in the implicit scheme,
+// 4.08 in second order, 4 in first), the longest chain of updates in a tile has R + C - 1 <= 17 of them
+// (2^37), and values start within [2^-64, 2^64].  Above it the tile is rescaled after every column.
 constexpr float kFdTileM = 1.0f;
 
 // One lane's row of the FD forward tape: its R node differences v (before the tile's update), the
