@@ -778,15 +778,15 @@ def main():
         il = torch.zeros(1, dtype=torch.int64, device=dev)
         ol = torch.empty(1, dtype=torch.float64, device=dev)
         cells_l = 16384 * 16384
-        t_grid = timed_steps(lambda: sk.sigkernel_pairs(Xl, Yl, il, il, compute="f32", out=ol), 2, 1)
-        # the oracle checks a pair of 4097-point prefixes, swept the same way (a ring of 8 blocks)
+        t_long = timed_steps(lambda: sk.sigkernel_pairs(Xl, Yl, il, il, compute="f32", out=ol), 2, 1)
+        # the oracle checks a pair of 4097-point prefixes, swept the same way (128 strips, a warp each)
         Xp, Yp = Xl[:, :4097].contiguous(), Yl[:, :4097].contiguous()
         op = sk.sigkernel_pairs(Xp, Yp, il, il, compute="f32").cpu().numpy()
         samples["long_prefix4097"] = dict(xs=[Xl_np[0, :4097]], ys=[Yl_np[0, :4097]], pa=[0], pb=[0],
                                           scheme="approx", N=DEGREE, lam=0, gpu=op)
         line["long_pair"] = {"workload": "1 pair of 16385-point Brownian paths, d=4, approx N=6, FP32: the pair's "
-                                         "512 strips swept by a ring of 32 co-resident 16-warp blocks",
-                             "cells": cells_l, "ms": t_grid, "cell_updates_per_s": cells_l / (t_grid / 1e3),
+                                         "512 strips swept by a warp each (strip chain)",
+                             "cells": cells_l, "ms": t_long, "cell_updates_per_s": cells_l / (t_long / 1e3),
                              "oracle_check": "a pair of 4097-point prefixes in the same strip chain"}
         del Xl, Yl
 
