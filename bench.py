@@ -129,6 +129,20 @@ NCU_TRAFFIC_RATIO = {"bwd_tape_kernel<float,6,false>": (2.270 + 0.185) / 2.402,
                      "fwd_poly_kernel<float,6,6,false,false,true,true>": (2.207 + 0.161) / 2.242}
 
 
+# Keys of the line that are printed as measured; the floats of the others to six digits.
+HEADLINE = ("value", "ms_per_step", "vs_baseline", "e2e", "clocks")
+
+
+def short_line(line):
+    def six(v):
+        if isinstance(v, float):
+            return float(f"{v:.6g}")
+        if isinstance(v, dict):
+            return {k: six(x) for k, x in v.items()}
+        return [six(x) for x in v] if isinstance(v, list) else v
+    return {k: v if k in HEADLINE else six(v) for k, v in line.items()}
+
+
 def parse():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -874,16 +888,18 @@ def main():
         def sig3(rep):
             return {L: {k: (round(v, 12) if k == "truth_check" else {o: float(f"{e:.3g}") for o, e in v.items()})
                         for k, v in row.items()} for L, row in rep["lengths"].items()}
-        line["accuracy"] = {"truth": "interpolation N=12, lambda=3, FP64 (checked against approximation N=16)",
-                            "unit": "MAPE in percent; keys: order N (approx, interp) or dyadic lambda (fd*)"}
+        study = {"truth": "interpolation N=12, lambda=3, FP64 (checked against approximation N=16)",
+                 "unit": "MAPE in percent; keys: order N (approx, interp) or dyadic lambda (fd*)"}
         for kind, lengths in (("sin", (10, 50, 100, 200)), ("brownian", (10, 50, 200))):
-            line["accuracy"][kind] = {c: sig3(accuracy.report(kind, lengths=lengths, compute=c))
-                                      for c in ("f64", "f32")}
+            study[kind] = {c: sig3(accuracy.report(kind, lengths=lengths, compute=c)) for c in ("f64", "f32")}
+        # twelve kilobytes of tables: beside the line, not in it (a line of 26 KB did not reach its reader whole)
+        print(json.dumps({"accuracy": study}), file=sys.stderr)
+        line["accuracy"] = "on stderr"
 
     if rank == 0:
         if "cpu" in args.parts:
             line["cpu_baseline"], line["mape_vs_fp64_oracle"] = cpu_baseline(X, Y, samples)
-        print(json.dumps(line))
+        print(json.dumps(short_line(line)))
     if dist is not None:
         dist.barrier()
         dist.destroy_process_group()
