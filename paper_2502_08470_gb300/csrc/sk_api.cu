@@ -383,6 +383,15 @@ size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 // Dynamic shared memory that every kernel may use without being allowed more: a block's 48 KB less
 // what a kernel declares statically (the strip chain's hand-off buffers).
 constexpr int kPlainSmem = 32 * 1024;
+// Allows a kernel the dynamic shared memory that a plan gives it.  The allowance is the kernel's, not the
+// plan's: a call plans several launches of one kernel before it makes them (the blocks of MMD^2, whose
+// sets may differ in length), and other threads plan theirs meanwhile, so it is never set to less than
+// what any plan may ask for (200 KB; a launch's own size alone decides how many blocks an SM takes).
+constexpr int kAllowSmem = 200 * 1024;
+cudaError_t allow_smem(const void* kern, int bytes) {
+    if (bytes <= kPlainSmem) return cudaSuccess;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, std::max(bytes, kAllowSmem));
+}
 // Bytes of precomputed M a forward holds at once (the chunk of items whose M the tensor cores
 // wrote before the chunk's sweep); a chunk is a whole number of the sweep's resident warps.
 constexpr size_t kMxBudget = size_t(8) << 30;
@@ -629,7 +638,7 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     };
     auto occupancy = [&](const void* k, int threads, int* per) -> int {
         const int sm = xsmem(threads);
-        if (sm > kPlainSmem) SK_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+        SK_CUDA(allow_smem(k, sm));
         SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per, k, threads, sm));
         return SK_OK;
     };
@@ -1042,7 +1051,7 @@ int run_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype, 
     }
     int64_t buf_cols = p.buf_cols;
     const int smem = p.smem_x;  // tiled-M x rows
-    if (smem > kPlainSmem) SK_CUDA(cudaFuncSetAttribute(p.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    SK_CUDA(allow_smem(p.kern, smem));
     const bool timed = (o->flags & SK_FLAG_TIME_KERNEL) != 0;
     if (timed) {
         if (!t_ev0) SK_CUDA(cudaEventCreate(&t_ev0));
@@ -1173,7 +1182,7 @@ int plan_backward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype
     int dev = 0, sms = 0, per_sm = 0;
     SK_CUDA(cudaGetDevice(&dev));
     SK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    SK_CUDA(cudaFuncSetAttribute(b.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, b.smem_bytes));
+    SK_CUDA(allow_smem(b.kern, b.smem_bytes));
     SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b.kern, p.threads, b.smem_bytes));
     if (per_sm < 1) return fail(SK_ERR_UNSUPPORTED, "adjoint kernel does not fit an SM (%d bytes shared)", b.smem_bytes);
     const int64_t want = (npairs + kFwdWarps - 1) / kFwdWarps;
@@ -1394,10 +1403,10 @@ int plan_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t 
     int dev = 0, sms = 0, per_sm = 0, cper_sm = 0;
     SK_CUDA(cudaGetDevice(&dev));
     SK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    SK_CUDA(cudaFuncSetAttribute(b.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, b.smem_bytes));
+    SK_CUDA(allow_smem(b.kern, b.smem_bytes));
     SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b.kern, p.threads, b.smem_bytes));
     if (per_sm < 1) return fail(SK_ERR_UNSUPPORTED, "adjoint kernel does not fit an SM");
-    SK_CUDA(cudaFuncSetAttribute(b.ckern, cudaFuncAttributeMaxDynamicSharedMemorySize, b.csmem));
+    SK_CUDA(allow_smem(b.ckern, b.csmem));
     SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cper_sm, b.ckern, kContractWarps * 32,
                                                           static_cast<size_t>(b.csmem)));
     if (cper_sm < 1) return fail(SK_ERR_UNSUPPORTED, "contraction kernel does not fit an SM");
@@ -1416,7 +1425,7 @@ int plan_backward_tape(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t 
         ((o->flags & SK_FLAG_STRIP_PIPELINE) || chain_pays(X, Y, points, o->dyadic, npairs, strips, max_cols,
                                                            sms, per_sm, p.T, true))) {
         int cper = 0;
-        SK_CUDA(cudaFuncSetAttribute(chain_kern, cudaFuncAttributeMaxDynamicSharedMemorySize, b.smem_bytes));
+        SK_CUDA(allow_smem(chain_kern, b.smem_bytes));
         SK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cper, chain_kern, p.threads, b.smem_bytes));
         size_t none = 0;
         if (cper >= 1 && plan_chain(b.chain, none, npairs, strips, max_cols, units, kChainAny)) {
