@@ -799,9 +799,14 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
 // Blocks of 128 threads over every element of a path set's rows: paths, and as many pieces of a path as
 // give the GPU about 16 such blocks per SM, at four elements a thread or more.
 int path_grid(const sk_paths* S, int width, dim3* grid) {
+    static std::atomic<int> known[64];  // SMs of each device, asked for once
     int dev = 0, sms = 0;
     SK_CUDA(cudaGetDevice(&dev));
-    SK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (dev < 64) sms = known[dev].load(std::memory_order_relaxed);
+    if (sms == 0) {
+        SK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        if (dev < 64) known[dev].store(sms, std::memory_order_relaxed);
+    }
     const int64_t x = std::min<int64_t>(S->count, 65535);
     const int64_t y = std::min<int64_t>((S->max_len * width + 511) / 512, std::max<int64_t>(16 * sms / x, 1) * 2);
     *grid = dim3(static_cast<unsigned>(x), static_cast<unsigned>(std::max<int64_t>(y, 1)));
@@ -1699,6 +1704,8 @@ int plan_mmd2_blocks(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t d
     m.os = *o;
     m.os.flags = (o->flags & (SK_FLAG_INCREMENTS | SK_FLAG_NO_SORT | SK_FLAG_TIME_KERNEL | SK_FLAG_STRIP_PIPELINE |
                               SK_FLAG_NO_STRIP_PIPELINE | SK_FLAG_NO_TILED_M | SK_FLAG_NO_TC)) | SK_FLAG_SYMMETRIC;
+    // (sets of one length each say that a block's pairs need no order; pooled, the two lengths meet)
+    if (pooled && A->max_len != Bp->max_len) m.os.flags &= ~SK_FLAG_NO_SORT;
     m.of = m.os;
     m.of.flags &= ~SK_FLAG_SYMMETRIC;
     m.pooled = pooled;

@@ -454,18 +454,13 @@ def sigkernel_backward_tape(tape, grad_out, X, Y=None, pair_a=None, pair_b=None,
     return gX, gY
 
 
-def _mmd_sort_flag(A: Paths, B: Paths) -> int:
-    """MMD^2 pairs the paths of both sets with one another: FLAG_NO_SORT when all of them are as long."""
-    return FLAG_NO_SORT if A.equal and B.equal and A.max_len == B.max_len else 0
-
-
 def sigkernel_mmd2(A, B, scheme="approx", degree=6, dyadic=0, compute="f64", unbiased=False, grads=False,
                    tensor_cores: bool = True):
     """MMD^2 between path sets A and B; returns (mmd2, [mean K_AA, mean K_BB, mean K_AB]) or, with
     ``grads``, also (dMMD2/dA rows, dMMD2/dB rows) as float64 CUDA tensors."""
     A, B = as_paths(A), as_paths(B)
     cA, cB = _cpaths(A), _cpaths(B)
-    opt = _options(scheme, degree, dyadic, compute, _flags(A, (FLAG_UNBIASED if unbiased else 0) | _mmd_sort_flag(A, B)
+    opt = _options(scheme, degree, dyadic, compute, _flags(A, (FLAG_UNBIASED if unbiased else 0) | _sort_flag(True, A, B)
                                                            | (0 if tensor_cores else FLAG_NO_TC)))
     ws = _workspace(OP_MMD2, cA, cB, A.d, 1 if grads else 0, opt)
     out = torch.empty(4, dtype=torch.float64, device="cuda")
@@ -506,7 +501,7 @@ def sigkernel_mmd2_test(A, B, permutations=1000, labels=None, seed=0, scheme="ap
     labels = _device_buffer(labels.contiguous(), "labels", torch.uint8, labels.shape[0] * (A.count + B.count))
     nperm = labels.shape[0]
     cA, cB = _cpaths(A), _cpaths(B)
-    opt = _options(scheme, degree, dyadic, compute, _flags(A, (FLAG_UNBIASED if unbiased else 0) | _mmd_sort_flag(A, B)))
+    opt = _options(scheme, degree, dyadic, compute, _flags(A, (FLAG_UNBIASED if unbiased else 0) | _sort_flag(True, A, B)))
     ws = _device_buffer(workspace, "workspace") if workspace is not None else \
         _workspace(OP_MMD2_TEST, cA, cB, A.d, nperm, opt)
     if out is None:
@@ -521,7 +516,7 @@ def sigkernel_mmd2_test(A, B, permutations=1000, labels=None, seed=0, scheme="ap
 def mmd2_test_workspace(A, B, nperm, scheme="approx", degree=6, dyadic=0, compute="f64", unbiased=False):
     """Device workspace of ``sigkernel_mmd2_test`` for these sets and relabelling count."""
     A, B = as_paths(A), as_paths(B)
-    opt = _options(scheme, degree, dyadic, compute, _flags(A, (FLAG_UNBIASED if unbiased else 0) | _mmd_sort_flag(A, B)))
+    opt = _options(scheme, degree, dyadic, compute, _flags(A, (FLAG_UNBIASED if unbiased else 0) | _sort_flag(True, A, B)))
     return _workspace(OP_MMD2_TEST, _cpaths(A), _cpaths(B), A.d, int(nperm), opt)
 
 

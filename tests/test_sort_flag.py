@@ -19,8 +19,6 @@ def test_flags():
                        (room, dense, 0), (room, room, 0)]:
         assert sk._sort_flag(True, X, Y) == flag
         assert sk._sort_flag(False, X, Y) == no
-    for A, B, flag in [(dense, equal, no), (dense, longer, 0), (ragged, dense, 0), (ragged, ragged, 0), (room, room, 0)]:
-        assert sk._mmd_sort_flag(A, B) == flag
 
 
 @pytest.mark.gpu
