@@ -796,17 +796,25 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     return SK_OK;
 }
 
+// SMs of the current device, asked for once.
+int sm_count(int* sms) {
+    static std::atomic<int> known[64];
+    int dev = 0;
+    SK_CUDA(cudaGetDevice(&dev));
+    *sms = dev < 64 ? known[dev].load(std::memory_order_relaxed) : 0;
+    if (*sms == 0) {
+        SK_CUDA(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev));
+        if (dev < 64) known[dev].store(*sms, std::memory_order_relaxed);
+    }
+    return SK_OK;
+}
+
 // Blocks of 128 threads over every element of a path set's rows: paths, and as many pieces of a path as
 // give the GPU about 16 such blocks per SM, at four elements a thread or more.
 int path_grid(const sk_paths* S, int width, dim3* grid) {
-    static std::atomic<int> known[64];  // SMs of each device, asked for once
-    int dev = 0, sms = 0;
-    SK_CUDA(cudaGetDevice(&dev));
-    if (dev < 64) sms = known[dev].load(std::memory_order_relaxed);
-    if (sms == 0) {
-        SK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        if (dev < 64) known[dev].store(sms, std::memory_order_relaxed);
-    }
+    int sms = 0;
+    const int rc = sm_count(&sms);
+    if (rc != SK_OK) return rc;
     const int64_t x = std::min<int64_t>(S->count, 65535);
     const int64_t y = std::min<int64_t>((S->max_len * width + 511) / 512, std::max<int64_t>(16 * sms / x, 1) * 2);
     *grid = dim3(static_cast<unsigned>(x), static_cast<unsigned>(std::max<int64_t>(y, 1)));
@@ -1784,11 +1792,26 @@ int plan_mmd2_blocks(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t d
     return SK_OK;
 }
 
+// Whether the values alone are those of so many pairs of one strip that three blocks fill the GPU as well as one
+// does (three waves of 32 warps per SM).  Pooled, every pair finds its two paths by a square root, which on
+// such short sweeps costs more than the two launch sets save: 150 + 150 paths of 14 and 12 points, d = 5,
+// 1.30 against 1.16 ms, 48 + 286 paths of 30 and 25 points 1.95 against 1.85; 100 + 150 of 65 points
+// 1.84 against 1.95.
+bool many_short_pairs(const sk_paths* A, const sk_paths* Bp, const sk_options* o) {
+    int sms = 0;
+    if (o->dyadic < 0 || o->dyadic > 5 || sm_count(&sms) != SK_OK) return false;  // (the plan reports what is wrong)
+    const int64_t points = (o->flags & SK_FLAG_INCREMENTS) ? 0 : 1;
+    const int64_t rows = std::max(A->max_len, Bp->max_len) - points;
+    const int64_t n = A->count + Bp->count;
+    return rows <= (32 >> o->dyadic) && n * (n + 1) / 2 > static_cast<int64_t>(3 * 32) * sms;
+}
+
 // chain_ok: strip chains, whose buffers may take much more than the rest, may be used.
 int plan_mmd2(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t dtype, const sk_options* o, bool grads,
               MmdPlan& m, bool chain_ok = true) {
-    if (A && Bp && A->count > 0 && Bp->count > 0 &&
-        4 * std::max(A->max_len, Bp->max_len) <= 5 * std::min(A->max_len, Bp->max_len)) {
+    if (A && Bp && o && A->count > 0 && Bp->count > 0 &&
+        4 * std::max(A->max_len, Bp->max_len) <= 5 * std::min(A->max_len, Bp->max_len) &&
+        (grads || !many_short_pairs(A, Bp, o))) {
         // (a pooled block that does not fit a plan, or whose tape chunks cannot fill the GPU, falls back)
         if (plan_mmd2_blocks(A, Bp, d, dtype, o, grads, true, m, chain_ok) == SK_OK && (!grads || m.tape[0])) return SK_OK;
         t_last_error.clear();

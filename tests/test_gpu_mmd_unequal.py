@@ -33,3 +33,19 @@ def test_gradients_of_unequal_sets(compute, tol, scheme, N, pa, pb, d):
     for got, parts in ((gA, (gaa, gab[0])), (gB, (gbb, gab[1]))):
         ref = sum(p.reshape(-1, d) for p in parts)
         assert (got - ref).abs().max() <= tol * max(p.abs().max() for p in parts)
+
+
+@pytest.mark.parametrize("compute,tol", [("f64", 1e-11), ("f32", 1e-5)])
+@pytest.mark.parametrize("na,nb", [(180, 20), (90, 90)])
+def test_values_of_many_short_pairs(compute, tol, na, nb):
+    """Sets on either side of the number of pairs from which on the value alone is taken from three blocks."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    A = torch.as_tensor(W.brownian(na, 12, 5, seed=793), dtype=torch.float64, device="cuda")
+    B = torch.as_tensor(W.brownian(nb, 14, 5, seed=794), dtype=torch.float64, device="cuda")
+    m, means = sk.sigkernel_mmd2(A, B, degree=6, compute=compute)
+    K = [sk.sigkernel_gram(X, Y, degree=6, compute="f64").mean() for X, Y in ((A, None), (B, None), (A, B))]
+    assert sk.device_status() == 0
+    for got, want in zip(means, K):
+        assert abs(got - want) <= tol * abs(want)
+    assert abs(m - (K[0] + K[1] - 2 * K[2])) <= 4 * tol * max(K)
