@@ -28,7 +28,8 @@ const void* fwd_approx_tape_mx_ptr_f32(int N);
 const void* fwd_approx_tape_ptr_f32(int N);
 const void* fwd_approx_tape_ptr_f32_mt(int N);
 const void* fwd_approx_tape_ptr_f64(int N);
-const void* fwd_fd_kernel_ptr(int T, int order, int lam, bool coop, bool tape = false, bool narrow = false);
+const void* fwd_fd_kernel_ptr(int T, int order, int lam, bool coop, bool tape = false, bool narrow = false,
+                              bool loop = false);  // loop: pipelined blocks, more than two chunks per row
 // Whether an FD call on paths of at most lx x ly increments takes one refined column a step (FP64, short
 // paths); tape: of the forward that records one and of its adjoint, whose layout depends on it.
 bool fd_narrow(int T, int order, int lam, int64_t lx, int64_t ly, int dpad, bool tape);
@@ -40,8 +41,8 @@ int fd_tape_row_elems(int T, int lam, bool narrow);
 int fd_tape_cols(int lam, bool narrow);  // refined columns per warp step
 // Shared memory of one warp of bwd_fd_tape_kernel (its ring of tape rows).
 int bwd_fd_ring_bytes(int T, int lam, bool narrow);
-const void* fwd_fd_coop_ptr(int T, int order, int lam);
-const void* fwd_fd_implicit_ptr(int T, int lam, bool coop);  // order 3
+const void* fwd_fd_coop_ptr(int T, int order, int lam, bool loop);
+const void* fwd_fd_implicit_ptr(int T, int lam, bool coop, bool loop = false);  // order 3
 const void* fwd_approx_ptr_f32(int N);
 const void* fwd_interp_ptr_f32(int N);
 const void* fwd_approx_chain_ptr_f32(int N);

@@ -77,7 +77,7 @@ __device__ __forceinline__ T fd_pow2(int e) {
 // warp's own when CW = 1).  In a block the hand-off is ordered by the progress words prog[]; a buffer
 // entry of strip g is overwritten by strip g + CW only after strip g + 1 has consumed it, because
 // strip g + CW depends on strip g + 1 through the strips in between.
-template <typename T, int ORDER, int R, int CW, bool TAPE = false, int C = fd_cols(R)>
+template <typename T, int ORDER, int R, int CW, bool TAPE = false, int C = fd_cols(R), bool LOOP = false>
 __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const PairDesc& P, int w, char* own_buf,
                                          const char* prev_buf, int* prog, int64_t buf_cols) {
     constexpr bool kRescale = std::is_same<T, float>::value;
@@ -167,7 +167,8 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
                     ea = eb;
                 }
             }
-            const T m = row_dot<T>(xrow, row_at(ybase, (jj * C) >> lam, row_bytes), L.nvec) * sub;
+            const T* yrow = row_at(ybase, (jj * C) >> lam, row_bytes);
+            const T m = (LOOP ? row_dot_loop<T>(xrow, yrow, L.nvec) : row_dot<T>(xrow, yrow, L.nvec)) * sub;
             if constexpr (TAPE) {  // the tile's inputs for the adjoint (fd_tape_row)
                 using V = typename Vec<T>::type;
                 constexpr int W = Vec<T>::W;
@@ -272,7 +273,11 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
 // unconstrained build took (2 blocks per SM).  The pipelined blocks keep their budget: capped at
 // two blocks per SM they ran slower (64 oscillatory pairs at lambda = 4: 30.1 against 22.1 ms).
 // TAPE (CW = 1): also record the forward tape of the FD adjoint (fd_tape_row, L.tape must be set).
-template <typename T, int ORDER, int R, int CW, bool TAPE = false, int C = fd_cols(R)>
+// LOOP: inner products by the loop alone.  Pipelined FP32 blocks at lambda = 0 with more than two chunks per
+// row take it: with the forms of one and two chunks beside it, the loop of three is not unrolled and its
+// loads wait for one another (6 x 36 pairs of about 1100 points, FD1, d = 10: 3.86 against 3.55 ms; d = 8,
+// two chunks: 3.29 against 3.48 ms).
+template <typename T, int ORDER, int R, int CW, bool TAPE = false, int C = fd_cols(R), bool LOOP = false>
 __global__ void __launch_bounds__((CW > 1 ? CW : kFwdWarps) * 32, (CW > 1 ? 1 : (TAPE ? 4 : 8)))
     fwd_fd_kernel(Launch L, int64_t buf_cols) {
     const int wib = threadIdx.x >> 5;
@@ -297,7 +302,7 @@ __global__ void __launch_bounds__((CW > 1 ? CW : kFwdWarps) * 32, (CW > 1 ? 1 : 
                 break;
             }
             if (!trivial_pair(L, item, P))
-                sweep_fd<T, ORDER, R, CW>(L, item, P, wib, own, block_base + ((wib + CW - 1) % CW) * L.scratch_stride,
+                sweep_fd<T, ORDER, R, CW, false, C, LOOP>(L, item, P, wib, own, block_base + ((wib + CW - 1) % CW) * L.scratch_stride,
                                           s_prog, buf_cols);
         }
     }

@@ -6,7 +6,9 @@ namespace sk {
 
 namespace {
 template <typename T, int ORDER>
-const void* fd_rows(int lam) {
+const void* fd_rows(int lam, bool loop) {
+    if constexpr (sizeof(T) == 4)
+        if (loop && lam == 0) return reinterpret_cast<const void*>(&fwd_fd_kernel<T, ORDER, 1, kCoopWarps, false, 1, true>);
     // rows per lane: R = min(2^lambda, 16) (a divisor of 2^lambda, so a lane's rows share a cell)
     switch (lam < 4 ? lam : 4) {
         case 0: return reinterpret_cast<const void*>(&fwd_fd_kernel<T, ORDER, 1, kCoopWarps>);
@@ -18,9 +20,9 @@ const void* fd_rows(int lam) {
 }
 }  // namespace
 
-const void* fwd_fd_coop_ptr(int T, int order, int lam) {
-    if (T == 1) return order == 2 ? fd_rows<float, 2>(lam) : fd_rows<float, 1>(lam);
-    return order == 2 ? fd_rows<double, 2>(lam) : fd_rows<double, 1>(lam);
+const void* fwd_fd_coop_ptr(int T, int order, int lam, bool loop) {
+    if (T == 1) return order == 2 ? fd_rows<float, 2>(lam, loop) : fd_rows<float, 1>(lam, loop);
+    return order == 2 ? fd_rows<double, 2>(lam, loop) : fd_rows<double, 1>(lam, loop);
 }
 
 }  // namespace sk

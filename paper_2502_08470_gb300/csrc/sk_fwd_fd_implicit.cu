@@ -7,7 +7,9 @@ namespace sk {
 
 namespace {
 template <typename T, int CW>
-const void* fd_rows(int lam) {
+const void* fd_rows(int lam, bool loop = false) {
+    if constexpr (sizeof(T) == 4 && CW > 1)
+        if (loop && lam == 0) return reinterpret_cast<const void*>(&fwd_fd_kernel<T, 3, 1, CW, false, 1, true>);
     // rows per lane: R = min(2^lambda, 16) (a divisor of 2^lambda, so a lane's rows share a cell)
     switch (lam < 4 ? lam : 4) {
         case 0: return reinterpret_cast<const void*>(&fwd_fd_kernel<T, 3, 1, CW>);
@@ -19,8 +21,8 @@ const void* fd_rows(int lam) {
 }
 }  // namespace
 
-const void* fwd_fd_implicit_ptr(int T, int lam, bool coop) {
-    if (T == 1) return coop ? fd_rows<float, kCoopWarps>(lam) : fd_rows<float, 1>(lam);
+const void* fwd_fd_implicit_ptr(int T, int lam, bool coop, bool loop) {
+    if (T == 1) return coop ? fd_rows<float, kCoopWarps>(lam, loop) : fd_rows<float, 1>(lam);
     return coop ? fd_rows<double, kCoopWarps>(lam) : fd_rows<double, 1>(lam);
 }
 
