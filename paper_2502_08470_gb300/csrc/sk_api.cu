@@ -1794,12 +1794,14 @@ int plan_mmd2_blocks(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t d
 }
 
 // Whether the values alone are those of so many pairs of one strip that three blocks fill the GPU as well as one
-// does (three waves of 32 warps per SM).  Pooled, every pair finds its two paths by a square root, which on
-// such short sweeps costs more than the two launch sets save: 150 + 150 paths of 14 and 12 points, d = 5,
-// 1.30 against 1.16 ms, 48 + 286 paths of 30 and 25 points 1.95 against 1.85; 100 + 150 of 65 points
-// 1.84 against 1.95.
-bool many_short_pairs(const sk_paths* A, const sk_paths* Bp, const sk_options* o) {
+// does (three waves of 32 warps per SM), with M from the tensor cores, whose kernel and the sweep that reads
+// it have least to do per pair.  Pooled, every pair finds its two paths by a square root, which then costs
+// more than the two launch sets save: 150 + 150 paths of 14 and 12 points, d = 5, 1.30 against 1.16 ms,
+// 48 + 286 paths of 30 and 25 points 1.95 against 1.85; 100 + 150 of 65 points 1.84 against 1.95.  Other
+// sweeps gain by pooling there too (44 + 249 of 12 points, d = 1, N = 4: 0.31 against 0.35 ms).
+bool many_short_pairs(const sk_paths* A, const sk_paths* Bp, const sk_options* o, int d) {
     int sms = 0;
+    if (o->scheme != SK_POLY_APPROX || o->compute != SK_COMPUTE_F32 || d <= 4 || d > 32 || (o->flags & SK_FLAG_NO_TC)) return false;
     if (o->dyadic < 0 || o->dyadic > 5 || sm_count(&sms) != SK_OK) return false;  // (the plan reports what is wrong)
     const int64_t points = (o->flags & SK_FLAG_INCREMENTS) ? 0 : 1;
     const int64_t rows = std::max(A->max_len, Bp->max_len) - points;
@@ -1812,7 +1814,7 @@ int plan_mmd2(const sk_paths* A, const sk_paths* Bp, int32_t d, int32_t dtype, c
               MmdPlan& m, bool chain_ok = true) {
     if (A && Bp && o && A->count > 0 && Bp->count > 0 &&
         4 * std::max(A->max_len, Bp->max_len) <= 5 * std::min(A->max_len, Bp->max_len) &&
-        (grads || !many_short_pairs(A, Bp, o))) {
+        (grads || !many_short_pairs(A, Bp, o, d))) {
         // (a pooled block that does not fit a plan, or whose tape chunks cannot fill the GPU, falls back)
         if (plan_mmd2_blocks(A, Bp, d, dtype, o, grads, true, m, chain_ok) == SK_OK && (!grads || m.tape[0])) return SK_OK;
         t_last_error.clear();
