@@ -592,7 +592,7 @@ int plan_forward(const sk_paths* X, const sk_paths* Y, int32_t d, int32_t dtype,
     auto kernel_for = [&](bool coop) -> const void* {  // coop: the FD schemes' pipelined blocks
         return poly ? fwd_poly_kernel_ptr(p.T, o->scheme == SK_POLY_INTERP, o->degree, false, p.mtile, tape)
                     : fwd_fd_kernel_ptr(p.T, fd_order(o), lam, coop, tape, narrow_fd(X, Y, o, p.T, p.dpad, tape),
-                                        p.nvec > 2);
+                                        coop ? p.nvec > 2 : p.nvec == 3);
     };
     p.kern = kernel_for(false);
     if (poly) {

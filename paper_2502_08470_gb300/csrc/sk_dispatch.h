@@ -29,7 +29,7 @@ const void* fwd_approx_tape_ptr_f32(int N);
 const void* fwd_approx_tape_ptr_f32_mt(int N);
 const void* fwd_approx_tape_ptr_f64(int N);
 const void* fwd_fd_kernel_ptr(int T, int order, int lam, bool coop, bool tape = false, bool narrow = false,
-                              bool loop = false);  // loop: pipelined blocks, more than two chunks per row
+                              bool loop = false);  // loop: inner products by the loop alone (FP32, lambda = 0)
 // Whether an FD call on paths of at most lx x ly increments takes one refined column a step (FP64, short
 // paths); tape: of the forward that records one and of its adjoint, whose layout depends on it.
 bool fd_narrow(int T, int order, int lam, int64_t lx, int64_t ly, int dpad, bool tape);

@@ -8,7 +8,9 @@ namespace sk {
 
 namespace {
 template <typename T, int ORDER>
-const void* fd_rows(int lam) {
+const void* fd_rows(int lam, bool loop = false) {
+    if constexpr (sizeof(T) == 4)
+        if (loop && lam == 0) return reinterpret_cast<const void*>(&fwd_fd_kernel<T, ORDER, 1, 1, false, 1, true>);
     // rows per lane: R = min(2^lambda, 16) (a divisor of 2^lambda, so a lane's rows share a cell)
     switch (lam < 4 ? lam : 4) {
         case 0: return reinterpret_cast<const void*>(&fwd_fd_kernel<T, ORDER, 1, 1>);
@@ -107,7 +109,7 @@ const void* fwd_fd_kernel_ptr(int T, int order, int lam, bool coop, bool tape, b
     if (narrow && !coop) return order == 3 ? fd_rows_narrow<3>(lam) : order == 2 ? fd_rows_narrow<2>(lam) : fd_rows_narrow<1>(lam);
     if (order == 3) return fwd_fd_implicit_ptr(T, lam, coop, loop);
     if (coop) return fwd_fd_coop_ptr(T, order, lam, loop);
-    if (T == 1) return order == 2 ? fd_rows<float, 2>(lam) : fd_rows<float, 1>(lam);
+    if (T == 1) return order == 2 ? fd_rows<float, 2>(lam, loop) : fd_rows<float, 1>(lam, loop);
     return order == 2 ? fd_rows<double, 2>(lam) : fd_rows<double, 1>(lam);
 }
 

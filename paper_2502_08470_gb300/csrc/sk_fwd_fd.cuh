@@ -273,10 +273,11 @@ __device__ __forceinline__ void sweep_fd(const Launch& L, int64_t item, const Pa
 // unconstrained build took (2 blocks per SM).  The pipelined blocks keep their budget: capped at
 // two blocks per SM they ran slower (64 oscillatory pairs at lambda = 4: 30.1 against 22.1 ms).
 // TAPE (CW = 1): also record the forward tape of the FD adjoint (fd_tape_row, L.tape must be set).
-// LOOP: inner products by the loop alone.  Pipelined FP32 blocks at lambda = 0 with more than two chunks per
-// row take it: with the forms of one and two chunks beside it, the loop of three is not unrolled and its
-// loads wait for one another (6 x 36 pairs of about 1100 points, FD1, d = 10: 3.86 against 3.55 ms; d = 8,
-// two chunks: 3.29 against 3.48 ms).
+// LOOP: inner products by the loop alone, at lambda = 0 in FP32, where with the forms of one and two chunks
+// beside it the loop of three is slower: pipelined blocks take it from three chunks on (6 x 36 pairs of
+// about 1100 points, FD1, d = 10: 3.86 against 3.55 ms; d = 8, two chunks: 3.29 against 3.48 ms), one warp
+// per pair for three (64 x 80 pairs of 129 points, d = 10, implicit: 0.75 against 0.70 ms, FD1 0.66 against
+// 0.60; with six chunks it loses, 1.52 against 1.69 ms).
 template <typename T, int ORDER, int R, int CW, bool TAPE = false, int C = fd_cols(R), bool LOOP = false>
 __global__ void __launch_bounds__((CW > 1 ? CW : kFwdWarps) * 32, (CW > 1 ? 1 : (TAPE ? 4 : 8)))
     fwd_fd_kernel(Launch L, int64_t buf_cols) {
@@ -298,7 +299,7 @@ __global__ void __launch_bounds__((CW > 1 ? CW : kFwdWarps) * 32, (CW > 1 ? 1 : 
             const int nstrips = P.lx > 0 ? static_cast<int>((((P.lx << L.lam) / R) + 31) >> 5) : 0;
             if (nstrips < L.coop_min_strips) {  // short pairs from here on: one warp each
                 if (wib == 0 && !trivial_pair(L, item, P))
-                    sweep_fd<T, ORDER, R, 1>(L, item, P, 0, own, own, nullptr, buf_cols);
+                    sweep_fd<T, ORDER, R, 1, false, C, LOOP>(L, item, P, 0, own, own, nullptr, buf_cols);
                 break;
             }
             if (!trivial_pair(L, item, P))
@@ -311,7 +312,7 @@ __global__ void __launch_bounds__((CW > 1 ? CW : kFwdWarps) * 32, (CW > 1 ? 1 : 
         if (item < 0) break;
         const PairDesc P = decode_pair(L, item);
         if (trivial_pair(L, item, P)) continue;
-        sweep_fd<T, ORDER, R, 1, TAPE, C>(L, item, P, 0, own, own, nullptr, buf_cols);
+        sweep_fd<T, ORDER, R, 1, TAPE, C, LOOP>(L, item, P, 0, own, own, nullptr, buf_cols);
     }
 }
 

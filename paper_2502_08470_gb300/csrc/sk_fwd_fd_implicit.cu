@@ -8,7 +8,7 @@ namespace sk {
 namespace {
 template <typename T, int CW>
 const void* fd_rows(int lam, bool loop = false) {
-    if constexpr (sizeof(T) == 4 && CW > 1)
+    if constexpr (sizeof(T) == 4)
         if (loop && lam == 0) return reinterpret_cast<const void*>(&fwd_fd_kernel<T, 3, 1, CW, false, 1, true>);
     // rows per lane: R = min(2^lambda, 16) (a divisor of 2^lambda, so a lane's rows share a cell)
     switch (lam < 4 ? lam : 4) {
@@ -22,7 +22,7 @@ const void* fd_rows(int lam, bool loop = false) {
 }  // namespace
 
 const void* fwd_fd_implicit_ptr(int T, int lam, bool coop, bool loop) {
-    if (T == 1) return coop ? fd_rows<float, kCoopWarps>(lam, loop) : fd_rows<float, 1>(lam);
+    if (T == 1) return coop ? fd_rows<float, kCoopWarps>(lam, loop) : fd_rows<float, 1>(lam, loop);
     return coop ? fd_rows<double, kCoopWarps>(lam) : fd_rows<double, 1>(lam);
 }
 
