@@ -377,6 +377,9 @@ template <typename T, int N, int NE, bool INTERP, bool MT, bool DMT = false, boo
 __device__ __forceinline__ void sweep_poly(const Launch& L, int64_t item, const PairDesc& P, char* own_buf,
                                            int64_t buf_cols, T* xstage) {
     constexpr bool kRescale = std::is_same<T, float>::value;
+    // FP64 cells of order 8 and more leave no room for the inner product's short forms (19 x 130 pairs of 29 and
+    // 26 points, d = 3: order 10 3.18 against 3.06 ms, order 11 3.84 against 3.67; order 7 the other way).
+    constexpr bool kLoopDot = std::is_same<T, double>::value && !INTERP && N >= 8;
     static_assert(!MX || (!MT && std::is_same<T, float>::value), "precomputed M: FP32");
     using V = typename Vec<T>::type;
     constexpr int W = Vec<T>::W;
@@ -488,6 +491,7 @@ __device__ __forceinline__ void sweep_poly(const Launch& L, int64_t item, const 
             M = active ? mcur.x : T(0);
             mcur = make_float4(mcur.y, mcur.z, mcur.w, 0.f);
         }
+        else if constexpr (kLoopDot) M = row_dot_loop<T>(xrow, row_at(ybase, jc >> lam, row_bytes), L.nvec) * sub;
         else M = row_dot<T>(xrow, row_at(ybase, jc >> lam, row_bytes), L.nvec) * sub;
         if constexpr (INTERP) {
             if (L.tape != nullptr) {
