@@ -535,9 +535,13 @@ bool chain_pays(const sk_paths* X, const sk_paths* Y, int64_t points, int lam, i
     const double rx = std::max(1.0, static_cast<double>(X->rows_total) / X->count - points) * (1 << lam);
     const double ry = std::max(1.0, static_cast<double>(Y->rows_total) / Y->count - points) * (1 << lam);
     const double total = static_cast<double>(npairs) * std::ceil(rx / 32.0) * std::max(ry, 32.0);
-    const double full = total / (static_cast<double>(sms * per_sm * kFwdWarps) / (T ? 2 : 4));
+    // (warps at full rate: in FP64 a block to an SM)
+    const double full = total / static_cast<double>(T ? sms * per_sm * kFwdWarps / 2 : sms * kFwdWarps);
     const double one = std::max(static_cast<double>(pair), full);
-    const double chained = std::max(static_cast<double>(cols + kChainLag * strips), 1.1 * full);
+    // a chained strip pays its own ramp of 31 steps; in FP64 the fill comes on top, in FP32 it hides behind the batch
+    const double all = 1.1 * full * (1.0 + 31.0 / std::max(ry, 32.0));
+    const double fill = static_cast<double>(kChainLag * strips);
+    const double chained = T ? std::max(static_cast<double>(cols) + fill, all) : std::max(static_cast<double>(cols), all) + fill;
     return chained < 0.9 * one;
 }
 
