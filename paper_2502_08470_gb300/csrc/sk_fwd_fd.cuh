@@ -33,7 +33,7 @@
 // 128 x 128 Gram of 129-point paths, d = 8, FP32, 6.24 -> 2.87 ms with 4 columns a step, then 302 warp
 // instructions a step (112 of them the 16 sub-cells) at 0.76 issued a cycle: bound by issue.  Inner
 // products without a loop (2.55 ms) and the row's index, test and increments kept over a strip instead
-// of formed each step (2.35 ms) took more of them out.  FD2, lambda = 1, 48 x 48 pairs, forward with
+// of formed each step (2.35 ms) took more of them out: 255 a step now, at the same rate.  FD2, lambda = 1, 48 x 48 pairs, forward with
 // tape and adjoint: 1.63 -> 1.02 ms with 2 columns a step, whose tape is half as long, now 0.91 ms.
 #pragma once
 
